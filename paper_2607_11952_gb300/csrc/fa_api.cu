@@ -280,7 +280,7 @@ fa_status fa_ctx_create(const fa_graph* g1, const fa_graph* g2,
       (st = dalloc(&c->intra2, (size_t)g2->d.nnz, acc)) != FA_OK ||
       (st = dalloc(&c->anc_ptr, (size_t)(n1 + 1), acc)) != FA_OK ||
       (st = dalloc(&c->anc_col, 1, acc)) != FA_OK ||
-      (st = dalloc(&c->err_part, (size_t)((n2 + 255) / 256), acc)) != FA_OK ||
+      (st = dalloc(&c->err_part, (size_t)col_finalize_max_blocks((int)n2), acc)) != FA_OK ||
       (st = dalloc(&c->ticket, 1, acc)) != FA_OK ||
       (st = dalloc(&c->err, 1, acc)) != FA_OK ||
       (st = dalloc(&c->diff, (size_t)kPlanDiffBlocks + 1, acc)) != FA_OK ||

@@ -149,6 +149,7 @@ fa_status launch_sweep(const SweepPlan& sp, int n1, int n2, int64_t ld,
                        float* log_u, float mu, float* colpart, int* status,
                        cudaStream_t s);
 int sweep_max_active_clusters(const SweepPlan& sp, bool bf16);
+int col_finalize_max_blocks(int n2);
 fa_status launch_col_finalize(int n2, int64_t ld, int G, const float* colpart,
                               const float* log_v_cur, float nu,
                               float* log_v_next, double* err_part,

@@ -17,7 +17,9 @@ namespace fa {
 
 constexpr int64_t kStaticMaxLd = 65536;            // padded columns
 constexpr int64_t kStaticColpart = int64_t(1) << 21;  // floats: 8 MiB
-constexpr int kStaticMaxBlocks = (int)((kStaticMaxLd + 255) / 256);
+// at least col_finalize_max_blocks(kStaticMaxLd): 32-column blocks below
+// 16,384 columns, 128-column blocks above, 512 of either at most
+constexpr int kStaticMaxBlocks = 512;
 
 // Partial column sums, one row of ld floats per row group of the sweep: at
 // most kStaticColpart / ld groups (32 at the largest ld), plus small counters.
@@ -102,6 +104,10 @@ extern "C" fa_status fa_sinkhorn_step_static(const void* K, int32_t dtype, int32
   if ((reinterpret_cast<uintptr_t>(K) & 15u) != 0) {
     set_error("fa_sinkhorn_step_static: K must be 16-byte aligned");
     return FA_ERR_ARG;
+  }
+  if (col_finalize_max_blocks(n2) > kStaticMaxBlocks) {
+    set_error("fa_sinkhorn_step_static: error partials exceed the static scratch");
+    return FA_ERR_UNSUPPORTED;
   }
   StaticScratch P;
   FA_TRY(static_scratch(&P));

@@ -822,72 +822,93 @@ int sweep_max_active_clusters(const SweepPlan& sp, bool bf16) {
 }
 
 // ------------------------------------------------------------ finalize
-// colsum_j = sum_g colpart[g][j] (in the order g = 0, 1, ..., G-1), column
-// marginal m_j = v_j colsum_j, err = sum_j |m_j - nu| in FP64 (deterministic
-// two-level reduction: per-block partials, summed by the last block in a
-// fixed order), and the next column scaling log v_j = log nu - log colsum_j.
-// Four columns per thread: colpart rows are read as 16-byte vectors (ld and
-// the column offsets passed in are multiples of 4); the log_v arrays are
-// read and written element by element (no alignment assumed).  v_j enters
-// the error through expf widened to FP64: the FP32 column sums already
-// carry a relative error of about G 2^-24, far above expf's.
+// colsum_j = sum_g colpart[g][j], column marginal m_j = v_j colsum_j, err =
+// sum_j |m_j - nu| in FP64 (deterministic two-level reduction: per-block
+// partials, summed by the last block in a fixed order), and the next column
+// scaling log v_j = log nu - log colsum_j.
+//
+// A block owns 4 LC columns: LC lanes side by side read one 16-byte vector
+// each of a partial row, and the block's 256 / LC thread groups take the
+// partial rows g, g + 256 / LC, ... in order (four in flight); the groups'
+// sums are then added in group order.  The kernel is bound by latency: G
+// partial rows (up to 600 at small sizes) must not be one thread's serial
+// chain, and few columns must still give enough blocks.  LC = 8 (32 columns,
+// 128-byte rows of 32 groups) below kFinNarrow columns, else LC = 32 (128
+// columns, 8 groups), where blocks are plenty.  Measured (GB300): 1,000
+// columns and 500 partial rows 44.8 -> 7.0 us, 10,000 and 296: 17.6 -> 7.0
+// us, 50,000 and 58: 13.5 -> 8.3 us, against four columns per thread and one
+// chain over all partial rows.
+// colpart rows are read as 16-byte vectors (ld and the column offsets passed
+// in are multiples of 4); the log_v arrays are read and written element by
+// element (no alignment assumed).  v_j enters the error through expf widened
+// to FP64: the FP32 column sums already carry a relative error of about
+// G 2^-24, far above expf's.
 constexpr int kFinThreads = 256;
-constexpr int kFinCols = 4;
+constexpr int kFinNarrow = 16384;
 
+template <int LC>
 __global__ void __launch_bounds__(kFinThreads) k_col_finalize(
     int n2, int64_t ld, int G, const float* __restrict__ colpart,
     const float* __restrict__ log_v_cur, float nu, float log_nu,
     float* __restrict__ log_v_next, double* __restrict__ err_part,
     unsigned* __restrict__ ticket, double* __restrict__ err_out,
     int* __restrict__ status) {
+  constexpr int C = 4 * LC, RG = kFinThreads / LC;
+  __shared__ __align__(16) float part[RG][C];
   __shared__ double sred[kFinThreads / 32];
   __shared__ bool last;
-  const int j = (blockIdx.x * kFinThreads + threadIdx.x) * kFinCols;
-  double e = 0.0;
-  if (j < n2) {
-    const float* p = colpart + j;
+  const int lc = threadIdx.x % LC, rg = threadIdx.x / LC;
+  const int jb = blockIdx.x * C;
+  {
     float4 cs = make_float4(0.f, 0.f, 0.f, 0.f);
-    int g = 0;
-    for (; g + 4 <= G; g += 4) {   // four rows in flight, added in row order
-      const float4 a0 = __ldcs(reinterpret_cast<const float4*>(p + (int64_t)g * ld));
-      const float4 a1 = __ldcs(reinterpret_cast<const float4*>(p + (int64_t)(g + 1) * ld));
-      const float4 a2 = __ldcs(reinterpret_cast<const float4*>(p + (int64_t)(g + 2) * ld));
-      const float4 a3 = __ldcs(reinterpret_cast<const float4*>(p + (int64_t)(g + 3) * ld));
-      cs.x += a0.x; cs.y += a0.y; cs.z += a0.z; cs.w += a0.w;
-      cs.x += a1.x; cs.y += a1.y; cs.z += a1.z; cs.w += a1.w;
-      cs.x += a2.x; cs.y += a2.y; cs.z += a2.z; cs.w += a2.w;
-      cs.x += a3.x; cs.y += a3.y; cs.z += a3.z; cs.w += a3.w;
-    }
-    for (; g < G; ++g) {
-      const float4 a = __ldcs(reinterpret_cast<const float4*>(p + (int64_t)g * ld));
-      cs.x += a.x; cs.y += a.y; cs.z += a.z; cs.w += a.w;
-    }
-    const float c4[kFinCols] = {cs.x, cs.y, cs.z, cs.w};
+    if (jb + 4 * lc < n2) {
+      const float* p = colpart + jb + 4 * lc;
+      int g = rg;
+      for (; g + 3 * RG < G; g += 4 * RG) {   // four rows in flight, added in row order
+        float4 a[4];
 #pragma unroll
-    for (int k = 0; k < kFinCols; ++k) {
-      const int jj = j + k;
-      if (jj >= n2) break;
-      const float c = c4[k];
-      if (log_v_cur) {
-        const double m = (double)expf(log_v_cur[jj]) * (double)c;
-        e += fabs(m - (double)nu);
+        for (int k = 0; k < 4; ++k)
+          a[k] = __ldcs(reinterpret_cast<const float4*>(p + (int64_t)(g + k * RG) * ld));
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          cs.x += a[k].x; cs.y += a[k].y; cs.z += a[k].z; cs.w += a[k].w;
+        }
       }
-      float lv;
-      if (c > 0.f && isfinite(c)) {
-        lv = log_nu - logf(c);
-      } else {
-        atomicOr(status, ST_NUMERIC);
-        lv = log_nu + 87.0f;   // keep finite; the status word reports it
+      for (; g < G; g += RG) {
+        const float4 a = __ldcs(reinterpret_cast<const float4*>(p + (int64_t)g * ld));
+        cs.x += a.x; cs.y += a.y; cs.z += a.z; cs.w += a.w;
       }
-      log_v_next[jj] = lv;
     }
+    *reinterpret_cast<float4*>(&part[rg][4 * lc]) = cs;
   }
-  for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
-  if ((threadIdx.x & 31) == 0) sred[threadIdx.x >> 5] = e;
+  __syncthreads();
+  double e = 0.0;
+  const int j = jb + (int)threadIdx.x;
+  if (threadIdx.x < C && j < n2) {
+    float c = 0.f;
+#pragma unroll
+    for (int r = 0; r < RG; ++r) c += part[r][threadIdx.x];
+    if (log_v_cur) {
+      const double m = (double)expf(log_v_cur[j]) * (double)c;
+      e = fabs(m - (double)nu);
+    }
+    float lv;
+    if (c > 0.f && isfinite(c)) {
+      lv = log_nu - logf(c);
+    } else {
+      atomicOr(status, ST_NUMERIC);
+      lv = log_nu + 87.0f;   // keep finite; the status word reports it
+    }
+    log_v_next[j] = lv;
+  }
+  if (threadIdx.x < C) {     // whole warps: C is a multiple of 32
+    for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+    if ((threadIdx.x & 31) == 0) sred[threadIdx.x >> 5] = e;
+  }
   __syncthreads();
   if (threadIdx.x == 0) {
     double t = 0.0;
-    for (int w = 0; w < kFinThreads / 32; ++w) t += sred[w];
+    for (int w = 0; w < C / 32; ++w) t += sred[w];
     err_part[blockIdx.x] = t;
     __threadfence();
     unsigned prev = atomicAdd(ticket, 1u);
@@ -914,9 +935,13 @@ __global__ void __launch_bounds__(kFinThreads) k_col_finalize(
   }
 }
 
-int col_finalize_blocks(int n2) {
-  const int per = kFinThreads * kFinCols;
-  return (n2 + per - 1) / per;
+static int col_finalize_cols(int n2) { return n2 < kFinNarrow ? 32 : 128; }
+
+// the most blocks (= entries of err_part) a finalisation of up to n2 columns
+// launches; a range narrower than kFinNarrow uses the narrow blocks
+int col_finalize_max_blocks(int n2) {
+  const int narrow = (std::min(n2, kFinNarrow) + 31) / 32, wide = (n2 + 127) / 128;
+  return std::max(narrow, wide);
 }
 
 fa_status launch_col_finalize(int n2, int64_t ld, int G, const float* colpart,
@@ -928,10 +953,14 @@ fa_status launch_col_finalize(int n2, int64_t ld, int G, const float* colpart,
     set_error("column finalisation: partial sums not 16-byte aligned");
     return FA_ERR_ARG;
   }
-  const int blocks = col_finalize_blocks(n2);
-  k_col_finalize<<<blocks, kFinThreads, 0, s>>>(
-      n2, ld, G, colpart, log_v_cur, nu, logf(nu), log_v_next, err_part,
-      ticket, err_out, status);
+  const int C = col_finalize_cols(n2);
+  const int blocks = (n2 + C - 1) / C;
+  if (C == 32)
+    k_col_finalize<8><<<blocks, kFinThreads, 0, s>>>(n2, ld, G, colpart, log_v_cur, nu, logf(nu),
+                                                     log_v_next, err_part, ticket, err_out, status);
+  else
+    k_col_finalize<32><<<blocks, kFinThreads, 0, s>>>(n2, ld, G, colpart, log_v_cur, nu, logf(nu),
+                                                      log_v_next, err_part, ticket, err_out, status);
   FA_LAUNCHED("k_col_finalize");
   return FA_OK;
 }
