@@ -82,7 +82,7 @@ namespace fa {
 // Host half of fa_build_graph (Algorithm 1, row normalisation): CSR of the symmetric adjacency
 // with columns ascending, values 1/deg_i (Abar) and 1/deg_k (Abar^T).
 struct HostCSR {
-  std::vector<int32_t> rp, col;
+  std::vector<int32_t> rp, col, row;
   std::vector<float> vr, vc;
   int32_t max_deg = 0;
   int64_t nnz = 0;
@@ -129,12 +129,14 @@ static fa_status csr_from_edges(const char* who, int32_t n, int64_t n_edges,
     h.col[pos[u]++] = v;
     h.col[pos[v]++] = u;
   }
+  h.row.resize(nnz);
   h.vr.resize(nnz);
   h.vc.resize(nnz);
   h.max_deg = 0;
   for (int i = 0; i < n; ++i) {
     h.max_deg = std::max(h.max_deg, deg[i]);
     for (int32_t e = h.rp[i]; e < h.rp[i + 1]; ++e) {
+      h.row[e] = i;
       h.vr[e] = 1.0f / (float)deg[i];
       h.vc[e] = 1.0f / (float)deg[h.col[e]];
     }
@@ -160,6 +162,7 @@ fa_status fa_build_graph(int32_t n, int64_t n_edges, const int32_t* src,
   fa_status st;
   if ((st = dalloc(&g->d.row_ptr, n + 1)) != FA_OK ||
       (st = dalloc(&g->d.col, nnz)) != FA_OK ||
+      (st = dalloc(&g->d.row, nnz)) != FA_OK ||
       (st = dalloc(&g->d.val_row, nnz)) != FA_OK ||
       (st = dalloc(&g->d.val_col, nnz)) != FA_OK) {
     fa_graph_destroy(g);
@@ -169,9 +172,10 @@ fa_status fa_build_graph(int32_t n, int64_t n_edges, const int32_t* src,
   cudaError_t e2 = nnz ? cudaMemcpy(g->d.col, h.col.data(), nnz * sizeof(int32_t), cudaMemcpyHostToDevice) : cudaSuccess;
   cudaError_t e3 = nnz ? cudaMemcpy(g->d.val_row, h.vr.data(), nnz * sizeof(float), cudaMemcpyHostToDevice) : cudaSuccess;
   cudaError_t e4 = nnz ? cudaMemcpy(g->d.val_col, h.vc.data(), nnz * sizeof(float), cudaMemcpyHostToDevice) : cudaSuccess;
-  if (e1 != cudaSuccess || e2 != cudaSuccess || e3 != cudaSuccess || e4 != cudaSuccess) {
+  cudaError_t e5 = nnz ? cudaMemcpy(g->d.row, h.row.data(), nnz * sizeof(int32_t), cudaMemcpyHostToDevice) : cudaSuccess;
+  if (e1 != cudaSuccess || e2 != cudaSuccess || e3 != cudaSuccess || e4 != cudaSuccess || e5 != cudaSuccess) {
     set_error("fa_build_graph: upload failed: %s",
-              cudaGetErrorString(e1 != cudaSuccess ? e1 : e2 != cudaSuccess ? e2 : e3 != cudaSuccess ? e3 : e4));
+              cudaGetErrorString(e1 != cudaSuccess ? e1 : e2 != cudaSuccess ? e2 : e3 != cudaSuccess ? e3 : e4 != cudaSuccess ? e4 : e5));
     fa_graph_destroy(g);
     return FA_ERR_CUDA;
   }
@@ -203,6 +207,7 @@ fa_status fa_graph_destroy(fa_graph* g) {
   if (!g) return FA_OK;
   dfree(g->d.row_ptr);
   dfree(g->d.col);
+  dfree(g->d.row);
   dfree(g->d.val_row);
   dfree(g->d.val_col);
   delete g;
@@ -219,7 +224,7 @@ fa_status fa_graph_info(const fa_graph* g, int32_t* n, int64_t* nnz) {
 // ------------------------------------------------------------ context
 fa_status fa_ctx_destroy(fa_ctx* c) {
   if (!c) return FA_OK;
-  dfree(c->Wt); dfree(c->X); dfree(c->rowmax_part); dfree(c->rowmax);
+  dfree(c->Wt); dfree(c->recs1); dfree(c->recs2); dfree(c->X); dfree(c->rowmax_part); dfree(c->rowmax);
   dfree(c->colpart); dfree(c->u_scale); dfree(c->v_scale);
   dfree(c->logv_buf[0]); dfree(c->logv_buf[1]);
   dfree(c->intra1); dfree(c->intra2); dfree(c->anc_ptr); dfree(c->anc_col);
@@ -268,6 +273,8 @@ fa_status fa_ctx_create(const fa_graph* g1, const fa_graph* g2,
   fa_status st;
   int64_t* acc = &c->ws_bytes;
   if ((st = dalloc(&c->Wt, (size_t)(n2 * ld1 * 2), acc)) != FA_OK ||
+      (st = dalloc(reinterpret_cast<char**>(&c->recs1), (size_t)g1->d.nnz * kEdgeRecBytes, acc)) != FA_OK ||
+      (st = dalloc(reinterpret_cast<char**>(&c->recs2), (size_t)g2->d.nnz * kEdgeRecBytes, acc)) != FA_OK ||
       (st = dalloc(&c->X, (size_t)(n1 * ld), acc)) != FA_OK ||
       (st = dalloc(&c->rowmax_part, (size_t)((ld / 64) * n1), acc)) != FA_OK ||
       (st = dalloc(&c->rowmax, (size_t)n1, acc)) != FA_OK ||
@@ -396,13 +403,15 @@ fa_status fa_node_cost(fa_ctx* c, const float* X1, const float* X2, int32_t d,
   }
   // Algorithm 1, RWR: R <- (1-beta) Abar R + beta R^(0), k_rwr times
   const float beta = c->p.beta;
+  FA_STEP(launch_edge_records(c->g1->d, c->g1->d.val_row, nullptr, nullptr, c->recs1, s));
+  FA_STEP(launch_edge_records(c->g2->d, c->g2->d.val_row, nullptr, nullptr, c->recs2, s));
   FA_STEP(launch_onehot(n1, L, ldr, da1, R1a, s));
   FA_STEP(launch_onehot(n2, L, ldr, da2, R2a, s));
   for (int t = 0; t < c->p.k_rwr; ++t) {
-    FA_STEP(launch_rwr_step(c->g1->d, L, ldr, beta, R1a, R1b, s));
+    FA_STEP(launch_rwr_step(c->g1->d, ldr, beta, c->recs1, R1a, R1b, s));
     FA_STEP(launch_add_onehot(L, ldr, da1, beta, R1b, s));
     std::swap(R1a, R1b);
-    FA_STEP(launch_rwr_step(c->g2->d, L, ldr, beta, R2a, R2b, s));
+    FA_STEP(launch_rwr_step(c->g2->d, ldr, beta, c->recs2, R2a, R2b, s));
     FA_STEP(launch_add_onehot(L, ldr, da2, beta, R2b, s));
     std::swap(R2a, R2b);
   }
@@ -434,10 +443,8 @@ fa_status fa_node_cost(fa_ctx* c, const float* X1, const float* X2, int32_t d,
   }
   // Algorithm 1, propagation (reading: A1bar C A2bar^T), k_prop times, as two SpMMs
   for (int t = 0; t < c->p.k_prop; ++t) {
-    FA_STEP(launch_spmm_left_T(c->g1->d, n2, c->ld, c->ld1, c->g1->d.val_row,
-                               nullptr, nullptr, C_node, false, c->Wt, s));
-    FA_STEP(launch_spmm_right_prop(c->g2->d, n1, c->ld1, c->g2->d.val_row,
-                                   c->Wt, C_node, c->ld, s));
+    FA_STEP(launch_spmm_T(c->g1->d, n2, c->ld, c->ld1, c->recs1, C_node, c->Wt, s));
+    FA_STEP(launch_spmm_T(c->g2->d, n1, c->ld1, c->ld, c->recs2, c->Wt, C_node, s));
   }
 #undef FA_STEP
   freeall();
@@ -458,12 +465,11 @@ fa_status fa_align_iter(fa_ctx* c, void* K, float* log_u, float* log_v,
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const bool bf16 = is_bf16(c);
   const int n1 = c->n1, n2 = c->n2;
-  FA_TRY(launch_exp_vec(n1, log_u, c->u_scale, s));
+  FA_TRY(launch_edge_records(c->g1->d, c->intra1, c->g1->d.val_col, log_u, c->recs1, s));
   FA_TRY(launch_exp_vec(n2, log_v, c->v_scale, s));
   // W = P1 T_prev for P1 in {C1, A1bar^T}; T_prev = diag(u) K diag(v): u is
   // folded into P1's column scale here and v into P2's below.
-  FA_TRY(launch_spmm_left_T(c->g1->d, n2, c->ld, c->ld1, c->intra1,
-                            c->g1->d.val_col, c->u_scale, K, bf16, c->Wt, s));
+  FA_TRY(launch_spmm_pair_T(c->g1->d, n2, c->ld, c->ld1, c->recs1, K, bf16, c->Wt, s));
   CostEpi ep;
   ep.C_node = C_node;
   ep.K_prev = K;

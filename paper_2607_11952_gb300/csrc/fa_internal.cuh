@@ -59,6 +59,7 @@ struct DevGraph {
   int64_t nnz = 0;
   int32_t* row_ptr = nullptr;   // n+1
   int32_t* col = nullptr;       // nnz, sorted per row
+  int32_t* row = nullptr;       // nnz: the row of each stored entry
   float* val_row = nullptr;     // Abar[i,k]   = 1/deg(i)
   float* val_col = nullptr;     // Abar^T[i,k] = 1/deg(k)
   int32_t max_deg = 0;
@@ -68,7 +69,10 @@ struct DevGraph {
 // (each returns FA_OK or FA_ERR_CUDA and counts its launches)
 
 // Phase 1
-fa_status launch_rwr_step(const DevGraph& g, int L, int64_t ldr, float beta,
+constexpr size_t kEdgeRecBytes = 16;      // one stored entry's record
+fa_status launch_edge_records(const DevGraph& g, const float* va, const float* vb,
+                              const float* log_scale, void* recs, cudaStream_t s);
+fa_status launch_rwr_step(const DevGraph& g, int64_t ldr, float beta, const void* recs,
                           const float* Rin, float* Rout, cudaStream_t s);
 fa_status launch_add_onehot(int L, int64_t ldr, const int32_t* nodes,
                             float value, float* R, cudaStream_t s);
@@ -106,13 +110,11 @@ struct CostEpi {
   float* X;                 // out: log of the unnormalised new kernel, n1 x ldo
   float* rowmax_part;       // out: [n2/64 tiles][n1] partial row maxima
 };
-fa_status launch_spmm_left_T(const DevGraph& g1, int n2, int64_t ldd,
-                             int64_t ldw, const float* va, const float* vb,
-                             const float* scale, const void* D, bool d_bf16,
-                             float* Wt, cudaStream_t s);
-fa_status launch_spmm_right_prop(const DevGraph& g2, int n1, int64_t ldw,
-                                 const float* qa, const float* Wt, float* C,
-                                 int64_t ldc, cudaStream_t s);
+fa_status launch_spmm_pair_T(const DevGraph& g1, int n2, int64_t ldd, int64_t ldw,
+                             const void* recs, const void* D, bool d_bf16, float* Wt,
+                             cudaStream_t s);
+fa_status launch_spmm_T(const DevGraph& g, int n_cols, int64_t ldd, int64_t ldw, const void* recs,
+                        const float* D, float* Wt, cudaStream_t s);
 fa_status launch_spmm_right_cost(const DevGraph& g2, int n1, int64_t ldw,
                                  int64_t ldo, const float* qa, const float* qb,
                                  const float* scale, const float* Wt,
@@ -196,6 +198,8 @@ struct fa_ctx {
   int device = 0;
   // workspaces (owned)
   float* Wt = nullptr;            // n2 x ld1 x 2 floats
+  void* recs1 = nullptr;          // nnz1 edge records
+  void* recs2 = nullptr;          // nnz2 edge records
   float* X = nullptr;             // n1 x ld floats
   float* rowmax_part = nullptr;   // (ld/64) x n1
   float* rowmax = nullptr;        // n1

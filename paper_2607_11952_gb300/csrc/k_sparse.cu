@@ -11,12 +11,15 @@
 // Storing the left product transposed turns both halves of the triple
 // product into coalesced row gathers; the CTA order keeps one column panel
 // of the gathered operand resident in L2 while every row tile uses it (the
-// GPU form of the paper's column-blocked SpMM, Section 3.4).
+// GPU form of the paper's column-blocked SpMM, Section 3.4).  The RWR, the
+// left products and the propagation's right product are one kernel
+// (k_spmm): a gather engine with a transposed or a row-major store.
 #include <math.h>
 
 #include <stdlib.h>
 
 #include "fa_internal.cuh"
+#include "sweep_dev.cuh"
 
 namespace fa {
 
@@ -48,57 +51,281 @@ fa_status launch_exp_vec(int n, const float* x, float* y, cudaStream_t s) {
   return FA_OK;
 }
 
-// ------------------------------------------------------------ RWR (Algorithm 1)
-// Rout[i,:] = (1-beta) sum_k Abar[i,k] Rin[k,:]; the beta R^(0) term is
-// added afterwards by k_add_onehot.  Column panels of 128 (one float4 per
-// lane), one warp per row, four neighbour gathers in flight; blockIdx.x runs
-// over rows first, so one panel of Rin (n x 128 floats) stays in L2 while
-// every row uses it instead of whole rows of Rin being re-read from HBM.
-__global__ void __launch_bounds__(256) k_rwr_step(
-    int n, int L, int64_t ldr, const int32_t* __restrict__ rp,
-    const int32_t* __restrict__ ci, const float* __restrict__ val, float c,
-    const float* __restrict__ Rin, float* __restrict__ Rout) {
-  const int row = blockIdx.x * 8 + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  const int64_t nv = ldr / 4;
-  const int64_t c4 = (int64_t)blockIdx.y * 32 + lane;
-  if (row >= n || c4 >= nv) return;
-  const int e0 = rp[row], e1 = rp[row + 1];
-  const float4* Rv = reinterpret_cast<const float4*>(Rin) + c4;
-  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-  int e = e0;
-  for (; e + 4 <= e1; e += 4) {
-    float w[4];
-    float4 r[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      w[u] = val[e + u];
-      r[u] = __ldg(Rv + (int64_t)ci[e + u] * nv);
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      acc.x = fmaf(w[u], r[u].x, acc.x); acc.y = fmaf(w[u], r[u].y, acc.y);
-      acc.z = fmaf(w[u], r[u].z, acc.z); acc.w = fmaf(w[u], r[u].w, acc.w);
-    }
-  }
-  for (; e < e1; ++e) {
-    const float w = val[e];
-    const float4 r = __ldg(Rv + (int64_t)ci[e] * nv);
-    acc.x = fmaf(w, r.x, acc.x); acc.y = fmaf(w, r.y, acc.y);
-    acc.z = fmaf(w, r.z, acc.z); acc.w = fmaf(w, r.w, acc.w);
-  }
-  acc.x *= c; acc.y *= c; acc.z *= c; acc.w *= c;
-  reinterpret_cast<float4*>(Rout + (int64_t)row * ldr)[c4] = acc;
+// ------------------------------------------------------------ edge records
+// One CSR edge as the gather kernels read it: the neighbour (the gathered
+// row), the output row and the weights of up to two value sets, already
+// multiplied by the neighbour's scaling exp(log_scale[nb]).  Built once per
+// product (16 bytes per stored entry) because every column panel of the
+// product, hundreds of them, reads every edge again.
+struct __align__(16) EdgeRec {
+  int nb, row;
+  float wa, wb;
+};
+
+__global__ void k_edge_records(int64_t nnz, const int32_t* __restrict__ ci,
+                               const int32_t* __restrict__ ri, const float* __restrict__ va,
+                               const float* __restrict__ vb, const float* __restrict__ log_scale,
+                               EdgeRec* __restrict__ out) {
+  const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (e >= nnz) return;
+  const int k = ci[e];
+  const float s = log_scale ? expf(log_scale[k]) : 1.f;
+  out[e] = EdgeRec{k, ri[e], va[e] * s, vb ? vb[e] * s : 0.f};
 }
 
-fa_status launch_rwr_step(const DevGraph& g, int L, int64_t ldr, float beta,
-                          const float* Rin, float* Rout, cudaStream_t s) {
-  if (g.n <= 0) return FA_OK;
-  dim3 grid((unsigned)((g.n + 7) / 8), (unsigned)((ldr / 4 + 31) / 32));
-  k_rwr_step<<<grid, 256, 0, s>>>(g.n, L, ldr, g.row_ptr, g.col, g.val_row, 1.0f - beta,
-                                  Rin, Rout);
-  FA_LAUNCHED("k_rwr_step");
+fa_status launch_edge_records(const DevGraph& g, const float* va, const float* vb,
+                              const float* log_scale, void* recs, cudaStream_t s) {
+  if (g.nnz <= 0) return FA_OK;
+  k_edge_records<<<(unsigned)((g.nnz + 255) / 256), 256, 0, s>>>(
+      g.nnz, g.col, g.row, va, vb, log_scale, static_cast<EdgeRec*>(recs));
+  FA_LAUNCHED("k_edge_records");
   return FA_OK;
+}
+
+__device__ __forceinline__ EdgeRec lds_edge(const EdgeRec* p) {
+  const int4 v = *reinterpret_cast<const int4*>(p);
+  return EdgeRec{v.x, v.y, __int_as_float(v.z), __int_as_float(v.w)};
+}
+
+// ------------------------------------------------------------ SpMM engine
+// out = P D for NV value sets of the sparse P (n rows) and the dense D, one
+// column panel of TJ = 32 V columns (V = 16 bytes of D per lane) and one
+// tile of TI rows of P per CTA.  OUT_T stores the product transposed, Wt[j,
+// i] (NV floats per element, TI consecutive i per column j); OUT_ROWS stores
+// alpha times it row-major.
+//
+// The tile's edges are one contiguous CSR range, split evenly over the NW
+// warps whatever the rows' degrees are: with one warp per row a hub row of
+// 700 neighbours kept its CTA's other warps idle.  A warp walks its edges
+// from the last to the first, the 512-byte gathers of kBatch of them in
+// flight while the kBatch before are added.  A row ends when the next edge's
+// row differs: its sum goes to the shared tile.  The last row of a warp may
+// have begun in an earlier warp's range; its sum is parked in place of the
+// warp's edge records and added in warp order, so every sum has a fixed
+// order and there are no atomics.  A lane's columns lie 32 apart in the tile
+// and its rows are RS = 1 (mod 32; 2 for tiles of 16 rows) apart: the
+// stores, lanes over columns, and the transposed reads, lanes over rows, are
+// free of bank conflicts.  blockIdx.x runs over row tiles first, so the panel
+// of D (rows x 512 bytes) stays in L2 while every tile gathers from it;
+// results are stored evict-first.
+//
+// What bounds it: the gathers of D's rows from L2, 512 bytes per edge and
+// panel, with what the resident warps keep in flight (random 512-byte
+// gathers alone, 128 KB in flight per SM: 20 TB/s).  Measured at 50,000 nodes
+// of average degree 10, exponent 2.1 (GB300), before -> after this form: Pass
+// A, BF16, two value sets, 25.1 -> 8.3 ms (50 GB of gathers, 25 GB of HBM);
+// propagation, FP32, left 12.4 -> 7.7 ms, right 25.3 -> 7.7 ms (100 GB of
+// gathers, 20 GB of HBM: 13 TB/s from L2); RWR step of 2,500 anchors 514 ->
+// 421 us.  Pass A at 10,000 nodes in FP32: 599 -> 363 us.
+// Tried on the same cases: batches of 4 (9.5 ms, 64 registers and fewer
+// warps) and 8 (12.0 ms); single gathers replaced one by one, 4 to 8 deep
+// (12 to 14 ms); gathers through a shared-memory ring by cp.async (10.3 ms,
+// and 13.4 ms for the propagation: every element crosses shared memory
+// twice); 16 warps (11.7 ms).  More resident warps beat deeper ones: the
+// shapes below take 4 warps where the tile is small enough for 9 CTAs per SM.
+enum { OUT_T = 0, OUT_ROWS = 1 };
+constexpr int kBatch = 2;         // gathers per batch, two batches in turn
+
+template <bool A16>
+__device__ __forceinline__ uint4 ldg16(const char* p) {
+  if constexpr (A16) {
+    return __ldg(reinterpret_cast<const uint4*>(p));
+  } else {                                       // 8-byte aligned operand
+    const uint2 a = __ldg(reinterpret_cast<const uint2*>(p));
+    const uint2 b = __ldg(reinterpret_cast<const uint2*>(p) + 1);
+    return make_uint4(a.x, a.y, b.x, b.y);
+  }
+}
+
+template <typename TD, int NV, int TI, int NW>
+struct SpmmShape {
+  static constexpr int V = 16 / (int)sizeof(TD);     // columns per lane
+  static constexpr int TJ = 32 * V;                  // columns per panel
+  static constexpr int F = TJ * NV;                  // floats per tile row
+  static constexpr int RS = F + 32 / TI;             // tile row stride
+  // per warp: 64 edge records, or a parked row
+  static constexpr int kWarpBytes = F * 4 > 64 * 16 ? F * 4 : 64 * 16;
+  static constexpr size_t smem = (size_t)NW * kWarpBytes + (size_t)TI * RS * sizeof(float);
+};
+
+template <typename TD, int NV, int TI, int NW, int MINB, int OUT, bool A16>
+__global__ void __launch_bounds__(32 * NW, MINB) k_spmm(
+    int n, int n_cols, int64_t ldd, int64_t ldo, const int32_t* __restrict__ rp,
+    const EdgeRec* __restrict__ recs, const TD* __restrict__ D, float alpha,
+    float* __restrict__ out) {
+  using Sh = SpmmShape<TD, NV, TI, NW>;
+  constexpr int V = Sh::V, TJ = Sh::TJ, F = Sh::F, RS = Sh::RS, V2 = V / 2;
+  constexpr int B = kBatch;
+  static_assert(32 % (2 * B) == 0, "records are staged 32 at a time");
+  extern __shared__ __align__(16) unsigned char sm_raw[];
+  float* tile = reinterpret_cast<float*>(sm_raw + NW * Sh::kWarpBytes);  // [TI][RS]
+  __shared__ int rps[TI + 1];
+  __shared__ int head_row[NW];
+  const int i0 = blockIdx.x * TI;
+  const int j0 = blockIdx.y * TJ;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  unsigned char* mine = sm_raw + warp * Sh::kWarpBytes;
+  for (int t = threadIdx.x; t <= TI; t += 32 * NW) rps[t] = rp[min(i0 + t, n)];
+  int cur = -1, cnt, eb;
+  f2_t acc[NV][V2];
+  auto clear = [&]() {
+#pragma unroll
+    for (int v = 0; v < NV; ++v)
+#pragma unroll
+      for (int k = 0; k < V2; ++k) acc[v][k] = pk2(0.f, 0.f);
+  };
+  auto store_row = [&](float* dst) {                  // column V lane + k at 32 k + lane
+#pragma unroll
+    for (int v = 0; v < NV; ++v)
+#pragma unroll
+      for (int k = 0; k < V2; ++k) {
+        const float2 a = upk2(acc[v][k]);
+        dst[v * TJ + (2 * k) * 32 + lane] = a.x;
+        dst[v * TJ + (2 * k + 1) * 32 + lane] = a.y;
+      }
+  };
+  {
+    const int E0 = rp[i0], len = rp[min(i0 + TI, n)] - E0;
+    eb = E0 + (int)((int64_t)len * warp / NW);
+    const int ee = E0 + (int)((int64_t)len * (warp + 1) / NW);
+    cnt = ee - eb;
+    // a lane past the operand's last column gathers the panel's first ones;
+    // its results are never stored
+    const int jl = j0 + lane * V < (int)ldd ? j0 + lane * V : j0;
+    const char* dcol = reinterpret_cast<const char*>(D + jl);
+    const uint32_t ldb = (uint32_t)(ldd * (int64_t)sizeof(TD));
+    EdgeRec* my = reinterpret_cast<EdgeRec*>(mine);   // edge ee - 1 - q in slot q & 63
+    const int4* rsrc = reinterpret_cast<const int4*>(recs) + (ee - 1 - lane);
+    int4 later;                                       // records of the batch after next
+    if (lane < cnt) *reinterpret_cast<int4*>(my + lane) = __ldg(rsrc);
+    if (32 + lane < cnt) *reinterpret_cast<int4*>(my + 32 + lane) = __ldg(rsrc - 32);
+    if (64 + lane < cnt) later = __ldg(rsrc - 64);
+    __syncwarp();
+    uint4 da[B], db[B];
+    // gathers of edges q .. q + B - 1; past the end the last edge's again
+    auto gather = [&](uint4 (&d)[B], int q) {
+#pragma unroll
+      for (int u = 0; u < B; ++u)
+        d[u] = ldg16<A16>(dcol + (uint64_t)(uint32_t)my[min(q + u, cnt - 1) & 63].nb * ldb);
+    };
+    auto add = [&](const uint4& d, int q) {
+      const EdgeRec er = lds_edge(my + (q & 63));
+      if (er.row != cur) {
+        if (cur >= 0) store_row(tile + (cur - i0) * RS);
+        clear();
+        cur = er.row;
+      }
+      f2_t x[V2];
+      pairs(d, x, TD());
+      const f2_t wa = pk2(er.wa, er.wa);
+#pragma unroll
+      for (int k = 0; k < V2; ++k) acc[0][k] = ffma2(wa, x[k], acc[0][k]);
+      if constexpr (NV == 2) {
+        const f2_t wb = pk2(er.wb, er.wb);
+#pragma unroll
+        for (int k = 0; k < V2; ++k) acc[NV - 1][k] = ffma2(wb, x[k], acc[NV - 1][k]);
+      }
+    };
+    if (cnt > 0) {
+      gather(da, 0);
+      int q = 0;
+      for (; q + 2 * B <= cnt; q += 2 * B) {
+        gather(db, q + B);
+#pragma unroll
+        for (int u = 0; u < B; ++u) add(da[u], q + u);
+        gather(da, q + 2 * B);
+#pragma unroll
+        for (int u = 0; u < B; ++u) add(db[u], q + B + u);
+        const int qn = q + 2 * B;
+        if ((qn & 31) == 0) {                         // a batch of 32 records is used up
+          __syncwarp();
+          if (qn + 32 + lane < cnt) *reinterpret_cast<int4*>(my + ((qn + 32 + lane) & 63)) = later;
+          if (qn + 64 + lane < cnt) later = __ldg(rsrc - (qn + 64));
+          __syncwarp();
+        }
+      }
+      if (q < cnt) {                                  // the last 1 .. 2 B - 1 edges
+        gather(db, q + B);
+#pragma unroll
+        for (int u = 0; u < B; ++u)
+          if (q + u < cnt) add(da[u], q + u);
+#pragma unroll
+        for (int u = 0; u < B; ++u)
+          if (q + B + u < cnt) add(db[u], q + B + u);
+      }
+    }
+  }
+  __syncthreads();                                    // rps; every warp is done with its records
+  {
+    const bool parked = cnt > 0 && rps[cur - i0] < eb;   // begun in an earlier warp's range
+    if (cnt > 0)
+      store_row(parked ? reinterpret_cast<float*>(mine) : tile + (cur - i0) * RS);
+    if (lane == 0) head_row[warp] = parked ? cur - i0 : -1;
+  }
+  __syncthreads();
+  // rows split between warps: the parked parts in warp order
+  for (int f = threadIdx.x; f < F; f += 32 * NW) {
+#pragma unroll
+    for (int w = 1; w < NW; ++w) {
+      const int r = head_row[w];
+      if (r >= 0) tile[r * RS + f] += reinterpret_cast<const float*>(sm_raw + w * Sh::kWarpBytes)[f];
+    }
+  }
+  __syncthreads();
+  if constexpr (OUT == OUT_T) {
+    // 32 / TI columns per pass (side by side in the tile), lanes over rows
+    constexpr int CP = 32 / TI;
+    const int r = lane % TI, hi = lane / TI;
+    const bool any = rps[r + 1] > rps[r];
+    const float* trow = tile + r * RS;
+    float* orow = out + (int64_t)(i0 + r) * NV;
+#pragma unroll 4
+    for (int p = warp * CP; p < TJ; p += NW * CP) {
+      const int f = p + hi, j = j0 + V * (f & 31) + (f >> 5);
+      if (j >= n_cols) continue;
+      if constexpr (NV == 1) {
+        __stcs(orow + (int64_t)j * ldo, any ? trow[f] : 0.f);
+      } else {
+        const float2 z = any ? make_float2(trow[f], trow[TJ + f]) : make_float2(0.f, 0.f);
+        __stcs(reinterpret_cast<float2*>(orow + (int64_t)j * ldo * 2), z);
+      }
+    }
+  } else {
+    // warp per row, a lane's V columns (NV = 1, V = 4)
+    static_assert(OUT == OUT_T || (NV == 1 && V == 4), "row-major store: one FP32 value set");
+    const int j = j0 + 4 * lane;
+    for (int r = warp; r < TI; r += NW) {
+      if (i0 + r >= n || j >= (int)ldo) continue;
+      const float* t = tile + r * RS + lane;
+      *reinterpret_cast<float4*>(out + (int64_t)(i0 + r) * ldo + j) =
+          rps[r + 1] > rps[r]
+              ? make_float4(alpha * t[0], alpha * t[32], alpha * t[64], alpha * t[96])
+              : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  }
+}
+
+template <typename TD, int NV, int TI, int NW, int MINB, int OUT, bool A16>
+static fa_status run_spmm(const DevGraph& g, int n_cols, int64_t panel_cols, int64_t ldd,
+                          int64_t ldo, const void* recs, const TD* D, float alpha, float* out,
+                          cudaStream_t s) {
+  using Sh = SpmmShape<TD, NV, TI, NW>;
+  auto* fn = &k_spmm<TD, NV, TI, NW, MINB, OUT, A16>;
+  FA_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sh::smem));
+  const dim3 grid((unsigned)((g.n + TI - 1) / TI), (unsigned)((panel_cols + Sh::TJ - 1) / Sh::TJ));
+  fn<<<grid, 32 * NW, Sh::smem, s>>>(g.n, n_cols, ldd, ldo, g.row_ptr,
+                                 static_cast<const EdgeRec*>(recs), D, alpha, out);
+  FA_LAUNCHED("k_spmm");
+  return FA_OK;
+}
+
+// ------------------------------------------------------------ RWR (Algorithm 1)
+// Rout[i,:] = (1-beta) sum_k Abar[i,k] Rin[k,:]; the beta R^(0) term is
+// added afterwards by k_add_onehot.  recs: Abar's records.
+fa_status launch_rwr_step(const DevGraph& g, int64_t ldr, float beta, const void* recs,
+                          const float* Rin, float* Rout, cudaStream_t s) {
+  return run_spmm<float, 1, 32, 8, 5, OUT_ROWS, true>(g, (int)ldr, ldr, ldr, ldr, recs, Rin,
+                                                      1.0f - beta, Rout, s);
 }
 
 // R[nodes[l], l] += value  (the beta R^(0) term; R^(0) is one-hot, Algorithm 1)
@@ -187,24 +414,34 @@ fa_status launch_normalize_rows(int n, int d, const float* X, int64_t ldx,
   return FA_OK;
 }
 
-// ------------------------------------------------------------ left SpMM
-// W^T[j, i] = sum_k P[i,k] s_k D[k, j]  for NV value sets P in {va, vb}.
-// CTA tile: 32 rows i x 128 columns j.  The tile's neighbour lists are one
-// contiguous CSR range [rp[i0], rp[i0+32]), split evenly over the 8 warps by
-// edge count, so high-degree rows are shared and warps finish together.  A
-// warp loads 32 edges at a time lane-parallel (neighbour k, weights times
-// s_k, output row by binary search in the tile's row pointers), broadcasts
-// them and keeps kGU row gathers of D[k, j0:j0+128] in flight (lane l:
-// columns 4l..4l+3, 256 B per gather in BF16, 512 B in FP32).  A finished row
-// goes to a shared-memory tile; a row split between warps (at most the first
-// and the last row of a warp's range) leaves one partial per warp in that
-// warp's head or tail slot, added in warp order afterwards, so the sums
-// are formed in a fixed order without atomics.  The tile is then stored
-// transposed, 32 consecutive i per column j (NV floats per element).  blockIdx.x runs over row tiles first, so all row
-// tiles of one 128-column panel of D run back-to-back and the panel
-// (n1 x 128 elements) stays in L2.
-constexpr int kGU = 8;     // gathers in flight per warp
+// ------------------------------------------------------------ products P D, stored transposed
+// Wt[j, i] = sum_k P[i,k] s_k D[k, j] for the two value sets of recs (Pass A:
+// C1 and A1bar^T on the plan's kernel).
+fa_status launch_spmm_pair_T(const DevGraph& g1, int n2, int64_t ldd, int64_t ldw,
+                             const void* recs, const void* D, bool d_bf16, float* Wt,
+                             cudaStream_t s) {
+  if (d_bf16) {
+    auto* Dp = static_cast<const __nv_bfloat16*>(D);
+    if ((reinterpret_cast<uintptr_t>(D) & 15u) == 0)
+      return run_spmm<__nv_bfloat16, 2, 16, 8, 4, OUT_T, true>(g1, n2, n2, ldd, ldw, recs, Dp,
+                                                               1.f, Wt, s);
+    return run_spmm<__nv_bfloat16, 2, 16, 8, 4, OUT_T, false>(g1, n2, n2, ldd, ldw, recs, Dp, 1.f,
+                                                              Wt, s);
+  }
+  return run_spmm<float, 2, 32, 8, 5, OUT_T, true>(g1, n2, n2, ldd, ldw, recs,
+                                                   static_cast<const float*>(D), 1.f, Wt, s);
+}
 
+// Wt[j, i] = sum_k P[i,k] D[k, j] for one value set and FP32 D: both halves
+// of the C_node propagation A1bar C A2bar^T (Algorithm 1) -- (A1bar C)^T,
+// then (A2bar (A1bar C)^T)^T.
+fa_status launch_spmm_T(const DevGraph& g, int n_cols, int64_t ldd, int64_t ldw, const void* recs,
+                        const float* D, float* Wt, cudaStream_t s) {
+  return run_spmm<float, 1, 32, 4, 9, OUT_T, true>(g, n_cols, n_cols, ldd, ldw, recs, D, 1.f, Wt,
+                                                   s);
+}
+
+// ------------------------------------------------------------ right SpMM with cost
 // Largest t in [0, n) with p[t] <= e, for p[0] <= e < p[n] (p nondecreasing).
 template <int N>
 __device__ __forceinline__ int seg_of(const int* p, int e) {
@@ -214,377 +451,6 @@ __device__ __forceinline__ int seg_of(const int* p, int e) {
     if (p[mid] <= e) lo = mid; else hi = mid;
   }
   return lo;
-}
-
-__device__ __forceinline__ float4 load_quad(const float* p) {
-  return __ldg(reinterpret_cast<const float4*>(p));
-}
-__device__ __forceinline__ float4 load_quad(const __nv_bfloat16* p) {
-  const uint2 u = __ldg(reinterpret_cast<const uint2*>(p));
-  return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xffff0000u),
-                     __uint_as_float(u.y << 16), __uint_as_float(u.y & 0xffff0000u));
-}
-
-// One CSR edge as a warp stages it: neighbour (gathered row), output row or
-// column within the tile, and the two weights times the neighbour's scaling.
-struct EdgeRec {
-  int nb, seg;
-  float wa, wb;
-};
-__device__ __forceinline__ EdgeRec lds_edge(const EdgeRec* p) {
-  const int4 v = *reinterpret_cast<const int4*>(p);
-  return EdgeRec{v.x, v.y, __int_as_float(v.z), __int_as_float(v.w)};
-}
-
-template <typename TD, int NV>
-__global__ void __launch_bounds__(256) k_spmm_left_T(
-    int n1, int n2, int64_t ldd, int64_t ldw, const int32_t* __restrict__ rp,
-    const int32_t* __restrict__ ci, const float* __restrict__ va,
-    const float* __restrict__ vb, const float* __restrict__ scale,
-    const TD* __restrict__ D, float* __restrict__ Wt) {
-  constexpr int TI = 32, TJ = 128;
-  // tile row stride (floats): a multiple of 4 so a lane's 4 columns are
-  // 16-byte stores; the +4 (+2 words per 64-bit read) spreads the banks of
-  // the transposed read over a half warp
-  constexpr int RS = TJ * NV + 4;
-  __shared__ __align__(16) float tile[TI * RS];
-  __shared__ __align__(16) float split_s[8][2][TJ * NV];   // [warp][head/tail][columns]
-  __shared__ int split_row[8][2];                          // row of each slot, -1 if unused
-  __shared__ __align__(16) EdgeRec edges[8][32];
-  __shared__ int rps[TI + 1];
-  const int i0 = blockIdx.x * TI;
-  const int j0 = blockIdx.y * TJ;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int t = threadIdx.x; t < TI * RS / 4; t += blockDim.x)
-    reinterpret_cast<float4*>(tile)[t] = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (threadIdx.x <= TI) rps[threadIdx.x] = rp[min(i0 + (int)threadIdx.x, n1)];
-  if (threadIdx.x < 16) split_row[threadIdx.x >> 1][threadIdx.x & 1] = -1;
-  __syncthreads();
-  {
-    const int E0 = rps[0], len = rps[TI] - E0;
-    const int eb = E0 + (int)((int64_t)len * warp / 8);
-    const int ee = E0 + (int)((int64_t)len * (warp + 1) / 8);
-    const TD* dcol = D + j0 + 4 * lane;
-    EdgeRec* my = edges[warp];
-    int cur = -1;
-    float acc[4][NV];
-#pragma unroll
-    for (int c = 0; c < 4; ++c)
-#pragma unroll
-      for (int v = 0; v < NV; ++v) acc[c][v] = 0.f;
-    auto flush = [&]() {
-      if (cur >= 0) {
-        float* dst = tile + cur * RS + 4 * lane * NV;
-        const bool starts_before = rps[cur] < eb, ends_after = rps[cur + 1] > ee;
-        if (starts_before || ends_after) {   // row split with another warp: a slot
-          const int slot = starts_before ? 0 : 1;
-          float* sp = &split_s[warp][slot][4 * lane * NV];
-#pragma unroll
-          for (int c = 0; c < 4; ++c)
-#pragma unroll
-            for (int v = 0; v < NV; ++v) sp[c * NV + v] = acc[c][v];
-          if (lane == 0) split_row[warp][slot] = cur;
-        } else if constexpr (NV == 2) {
-          reinterpret_cast<float4*>(dst)[0] = make_float4(acc[0][0], acc[0][1], acc[1][0], acc[1][1]);
-          reinterpret_cast<float4*>(dst)[1] = make_float4(acc[2][0], acc[2][1], acc[3][0], acc[3][1]);
-        } else {
-          reinterpret_cast<float4*>(dst)[0] = make_float4(acc[0][0], acc[1][0], acc[2][0], acc[3][0]);
-        }
-      }
-#pragma unroll
-      for (int c = 0; c < 4; ++c)
-#pragma unroll
-        for (int v = 0; v < NV; ++v) acc[c][v] = 0.f;
-    };
-    for (int base = eb; base < ee; base += 32) {
-      const int e = base + lane;
-      if (e < ee) {
-        const int k = ci[e];
-        const float sk = scale ? scale[k] : 1.f;
-        my[lane] = EdgeRec{k, seg_of<TI>(rps, e), va[e] * sk, NV == 2 ? vb[e] * sk : 0.f};
-      }
-      __syncwarp();
-      const int cnt = min(32, ee - base);
-      for (int u = 0; u < cnt; u += kGU) {
-        float4 d[kGU];
-#pragma unroll
-        for (int g = 0; g < kGU; ++g)
-          if (u + g < cnt) d[g] = load_quad(dcol + (int64_t)my[u + g].nb * ldd);
-#pragma unroll
-        for (int g = 0; g < kGU; ++g) {
-          if (u + g < cnt) {
-            const EdgeRec er = lds_edge(&my[u + g]);
-            if (er.seg != cur) {
-              flush();
-              cur = er.seg;
-            }
-            const float dv[4] = {d[g].x, d[g].y, d[g].z, d[g].w};
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-              acc[c][0] = fmaf(er.wa, dv[c], acc[c][0]);
-              if constexpr (NV == 2) acc[c][NV - 1] = fmaf(er.wb, dv[c], acc[c][NV - 1]);
-            }
-          }
-        }
-      }
-      __syncwarp();
-    }
-    flush();
-  }
-  __syncthreads();
-  // split rows: the warps' partials in warp order (head before tail)
-  for (int k = threadIdx.x; k < TJ * NV; k += blockDim.x) {
-    int row = -1;
-    float z = 0.f;
-    for (int w = 0; w < 8; ++w) {
-#pragma unroll
-      for (int sl = 0; sl < 2; ++sl) {
-        const int r = split_row[w][sl];
-        if (r < 0) continue;
-        if (r != row) {
-          if (row >= 0) tile[row * RS + k] = z;
-          row = r;
-          z = 0.f;
-        }
-        z += split_s[w][sl][k];
-      }
-    }
-    if (row >= 0) tile[row * RS + k] = z;
-  }
-  __syncthreads();
-  // transposed store: warp w writes columns c = w, w+8, ...; lane = row
-  for (int c = warp; c < TJ; c += 8) {
-    const int j = j0 + c;
-    if (j >= n2) break;
-    if constexpr (NV == 1) {
-      Wt[(int64_t)j * ldw + i0 + lane] = tile[lane * RS + c];
-    } else {
-      reinterpret_cast<float2*>(Wt + ((int64_t)j * ldw + i0) * 2)[lane] =
-          *reinterpret_cast<const float2*>(&tile[lane * RS + 2 * c]);
-    }
-  }
-}
-
-template <int NV> struct VecF;
-template <> struct VecF<1> { using T = float; };
-template <> struct VecF<2> { using T = float2; };
-
-// Row form of the left product, transposed store: CTA tile of 32 rows i by
-// 128 columns j; warp per row (4 rows per warp in turn), lane l covers
-// columns 4l .. 4l+3 of the tile, and kRowGathers neighbour rows
-// D[k, j0:j0+128] are in flight per warp (8 B per lane and gather in BF16,
-// 16 B in FP32).  Each output sums its row's edges in CSR order, so the
-// result does not depend on the tile shape.  Used for Pass A's two value
-// sets; FA_PASSA_ROWS=1 selects it for one value set too.
-constexpr int kRowGathers = 8;
-
-template <typename TD, int NV, int MINB>
-__global__ void __launch_bounds__(256, MINB) k_spmm_left_T_rows(
-    int n1, int n2, int64_t ldd, int64_t ldw, const int32_t* __restrict__ rp,
-    const int32_t* __restrict__ ci, const float* __restrict__ va,
-    const float* __restrict__ vb, const float* __restrict__ scale,
-    const TD* __restrict__ D, float* __restrict__ Wt) {
-  constexpr int TI = 32, TJ = 128, PAD = (NV == 1) ? 1 : 2, NG = kRowGathers;
-  __shared__ float tile[TI][TJ * NV + PAD];
-  const int i0 = blockIdx.x * TI;
-  const int j0 = blockIdx.y * TJ;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const TD* dcol = D + j0 + 4 * lane;
-#pragma unroll 1
-  for (int rr = 0; rr < 4; ++rr) {
-    const int r = warp * 4 + rr;
-    const int i = i0 + r;
-    float acc[4][NV];
-#pragma unroll
-    for (int c = 0; c < 4; ++c)
-#pragma unroll
-      for (int v = 0; v < NV; ++v) acc[c][v] = 0.f;
-    if (i < n1) {
-      const int e0 = rp[i], e1 = rp[i + 1];
-      int e = e0;
-      for (; e + NG <= e1; e += NG) {
-        int k[NG];
-        float4 d[NG];
-        float w[NG], x[NG];
-#pragma unroll
-        for (int u = 0; u < NG; ++u) k[u] = ci[e + u];
-#pragma unroll
-        for (int u = 0; u < NG; ++u) d[u] = load_quad(dcol + (int64_t)k[u] * ldd);
-#pragma unroll
-        for (int u = 0; u < NG; ++u) {
-          const float su = scale ? scale[k[u]] : 1.f;
-          w[u] = va[e + u] * su;
-          x[u] = NV == 2 ? vb[e + u] * su : 0.f;
-        }
-#pragma unroll
-        for (int u = 0; u < NG; ++u) {
-          const float dv[4] = {d[u].x, d[u].y, d[u].z, d[u].w};
-#pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            acc[c][0] = fmaf(w[u], dv[c], acc[c][0]);
-            if (NV == 2) acc[c][NV - 1] = fmaf(x[u], dv[c], acc[c][NV - 1]);
-          }
-        }
-      }
-      for (; e < e1; ++e) {
-        const int k0 = ci[e];
-        const float s0 = scale ? scale[k0] : 1.f;
-        const float4 d0 = load_quad(dcol + (int64_t)k0 * ldd);
-        const float dv[4] = {d0.x, d0.y, d0.z, d0.w};
-        const float w0 = va[e] * s0;
-        const float x0 = NV == 2 ? vb[e] * s0 : 0.f;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          acc[c][0] = fmaf(w0, dv[c], acc[c][0]);
-          if (NV == 2) acc[c][NV - 1] = fmaf(x0, dv[c], acc[c][NV - 1]);
-        }
-      }
-    }
-#pragma unroll
-    for (int c = 0; c < 4; ++c)
-#pragma unroll
-      for (int v = 0; v < NV; ++v) tile[r][(4 * lane + c) * NV + v] = acc[c][v];
-  }
-  __syncthreads();
-  // transposed store: warp w writes columns c = w, w+8, ...; lane = row
-  using VT = typename VecF<NV>::T;
-  for (int c = warp; c < TJ; c += 8) {
-    const int j = j0 + c;
-    if (j >= n2) break;
-    VT* dst = reinterpret_cast<VT*>(Wt + ((int64_t)j * ldw + i0) * NV);
-    if constexpr (NV == 1) {
-      dst[lane] = tile[lane][c];
-    } else {
-      dst[lane] = make_float2(tile[lane][c * 2], tile[lane][c * 2 + 1]);
-    }
-  }
-}
-
-fa_status launch_spmm_left_T(const DevGraph& g1, int n2, int64_t ldd,
-                             int64_t ldw, const float* va, const float* vb,
-                             const float* scale, const void* D, bool d_bf16,
-                             float* Wt, cudaStream_t s) {
-  const bool two = vb != nullptr;
-  // measured at 50k on GB300: the row-per-warp form is faster for the two
-  // value sets of Pass A in BF16 (14 vs 22 ms) and takes them always; for
-  // one value set (propagation) the forms were equal and FA_PASSA_ROWS=1
-  // selects the row form
-  static const int form = [] {
-    const char* v = getenv("FA_PASSA_ROWS");
-    return v ? atoi(v) : -1;
-  }();
-  if (form == 1 || two) {
-    dim3 g2d((unsigned)((g1.n + 31) / 32), (unsigned)((n2 + 127) / 128));
-    // 4 CTAs per SM (64 registers, a 32-byte spill in the BF16 two-set
-    // form) measured 48.7 ms per 50k outer iteration against 49.4 ms for 3
-    // (80 registers); FA_PASSA_MINB=3 selects 3 (tuning)
-    const char* mb = getenv("FA_PASSA_MINB");
-    const bool four = !(mb && atoi(mb) == 3);
-#define FA_PA(T, NVV)                                                                      \
-    if (four) k_spmm_left_T_rows<T, NVV, 4><<<g2d, 256, 0, s>>>(g1.n, n2, ldd, ldw, g1.row_ptr, \
-                                                                g1.col, va, vb, scale, Dp, Wt); \
-    else k_spmm_left_T_rows<T, NVV, 3><<<g2d, 256, 0, s>>>(g1.n, n2, ldd, ldw, g1.row_ptr,      \
-                                                           g1.col, va, vb, scale, Dp, Wt);
-    if (d_bf16) {
-      auto* Dp = static_cast<const __nv_bfloat16*>(D);
-      if (two) { FA_PA(__nv_bfloat16, 2) } else { FA_PA(__nv_bfloat16, 1) }
-    } else {
-      auto* Dp = static_cast<const float*>(D);
-      if (two) { FA_PA(float, 2) } else { FA_PA(float, 1) }
-    }
-#undef FA_PA
-    FA_LAUNCHED("k_spmm_left_T_rows");
-    return FA_OK;
-  }
-  dim3 grid((unsigned)((g1.n + 31) / 32), (unsigned)((n2 + 127) / 128));
-  if (d_bf16)
-    k_spmm_left_T<__nv_bfloat16, 1><<<grid, 256, 0, s>>>(g1.n, n2, ldd, ldw, g1.row_ptr, g1.col, va, vb, scale,
-                                                         static_cast<const __nv_bfloat16*>(D), Wt);
-  else
-    k_spmm_left_T<float, 1><<<grid, 256, 0, s>>>(g1.n, n2, ldd, ldw, g1.row_ptr, g1.col, va, vb, scale,
-                                                 static_cast<const float*>(D), Wt);
-  FA_LAUNCHED("k_spmm_left_T");
-  return FA_OK;
-}
-
-// ------------------------------------------------------------ right SpMM
-// Z[i, j] = sum_{l in N2(j)} Q[j,l] s_l W^T[l, i].  CTA tile: 64 columns j x
-// 32 rows i; warp w owns columns j0+8w..j0+8w+7, lane = row offset, so each
-// neighbour l is one coalesced 128/256-byte gather of W^T[l, i0:i0+32] and
-// every lane ends up holding 8 consecutive outputs of its own row -- the
-// epilogue needs no transpose.  blockIdx.x runs over column tiles first so
-// the W^T panel of one row tile (n2 x 32 elements) stays in L2.
-template <int NV>
-__device__ __forceinline__ void right_accumulate(
-    int j, int n2, int64_t ldw, int i0, int lane,
-    const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
-    const float* __restrict__ qa, const float* __restrict__ qb,
-    const float* __restrict__ scale, const float* __restrict__ Wt,
-    float& za, float& zb) {
-  za = 0.f;
-  zb = 0.f;
-  if (j >= n2) return;
-  const int e0 = rp[j], e1 = rp[j + 1];
-  const float* base = Wt + (int64_t)(i0 + lane) * NV;
-  int e = e0;
-  for (; e + 2 <= e1; e += 2) {
-    const int l0 = ci[e], l1 = ci[e + 1];
-    const float s0 = scale ? scale[l0] : 1.f, s1 = scale ? scale[l1] : 1.f;
-    if constexpr (NV == 1) {
-      float w0 = __ldg(base + (int64_t)l0 * ldw);
-      float w1 = __ldg(base + (int64_t)l1 * ldw);
-      za += qa[e] * s0 * w0 + qa[e + 1] * s1 * w1;
-    } else {
-      float2 w0 = __ldg(reinterpret_cast<const float2*>(base + (int64_t)l0 * ldw * 2));
-      float2 w1 = __ldg(reinterpret_cast<const float2*>(base + (int64_t)l1 * ldw * 2));
-      za += qa[e] * s0 * w0.x + qa[e + 1] * s1 * w1.x;
-      zb += qb[e] * s0 * w0.y + qb[e + 1] * s1 * w1.y;
-    }
-  }
-  for (; e < e1; ++e) {
-    const int l0 = ci[e];
-    const float s0 = scale ? scale[l0] : 1.f;
-    if constexpr (NV == 1) {
-      za += qa[e] * s0 * __ldg(base + (int64_t)l0 * ldw);
-    } else {
-      float2 w0 = __ldg(reinterpret_cast<const float2*>(base + (int64_t)l0 * ldw * 2));
-      za += qa[e] * s0 * w0.x;
-      zb += qb[e] * s0 * w0.y;
-    }
-  }
-}
-
-// C_node propagation (Algorithm 1): plain store of Z.
-__global__ void __launch_bounds__(256) k_spmm_right_prop(
-    int n1, int n2, int64_t ldw, const int32_t* __restrict__ rp,
-    const int32_t* __restrict__ ci, const float* __restrict__ qa,
-    const float* __restrict__ Wt, float* __restrict__ C, int64_t ldc) {
-  const int j0 = blockIdx.x * 64, i0 = blockIdx.y * 32;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int jb = j0 + warp * 8;
-  float z[8];
-#pragma unroll
-  for (int q = 0; q < 8; ++q) {
-    float zb;
-    right_accumulate<1>(jb + q, n2, ldw, i0, lane, rp, ci, qa, nullptr,
-                        nullptr, Wt, z[q], zb);
-  }
-  const int i = i0 + lane;
-  if (i < n1) {
-    float4* dst = reinterpret_cast<float4*>(C + (int64_t)i * ldc + jb);
-    dst[0] = make_float4(z[0], z[1], z[2], z[3]);
-    dst[1] = make_float4(z[4], z[5], z[6], z[7]);
-  }
-}
-
-fa_status launch_spmm_right_prop(const DevGraph& g2, int n1, int64_t ldw,
-                                 const float* qa, const float* Wt, float* C,
-                                 int64_t ldc, cudaStream_t s) {
-  dim3 grid((unsigned)(ldc / 64), (unsigned)((n1 + 31) / 32));
-  k_spmm_right_prop<<<grid, 256, 0, s>>>(n1, g2.n, ldw, g2.row_ptr, g2.col,
-                                         qa, Wt, C, ldc);
-  FA_LAUNCHED("k_spmm_right_prop");
-  return FA_OK;
 }
 
 // Cost assembly + log Gibbs kernel (Phase 2 of Algorithm 1, Eq. 2, proximal step):
@@ -683,9 +549,9 @@ __global__ void __launch_bounds__(256, MINB) k_spmm_right_cost(
         for (int k = 0; k < GU; ++k) {
           if (u + k < cnt) {
             const EdgeRec er = lds_edge(&my[u + k]);
-            if (er.seg != cur) {
+            if (er.row != cur) {
               flush();
-              cur = er.seg;
+              cur = er.row;
             }
             a0 = fmaf(er.wa, w[k].x, a0);
             b0 = fmaf(er.wb, w[k].y, b0);
