@@ -466,7 +466,7 @@ fa_status fa_align_iter(fa_ctx* c, void* K, float* log_u, float* log_v,
   const bool bf16 = is_bf16(c);
   const int n1 = c->n1, n2 = c->n2;
   FA_TRY(launch_edge_records(c->g1->d, c->intra1, c->g1->d.val_col, log_u, c->recs1, s));
-  FA_TRY(launch_exp_vec(n2, log_v, c->v_scale, s));
+  FA_TRY(launch_edge_records(c->g2->d, c->intra2, c->g2->d.val_col, log_v, c->recs2, s));
   // W = P1 T_prev for P1 in {C1, A1bar^T}; T_prev = diag(u) K diag(v): u is
   // folded into P1's column scale here and v into P2's below.
   FA_TRY(launch_spmm_pair_T(c->g1->d, n2, c->ld, c->ld1, c->recs1, K, bf16, c->Wt, s));
@@ -487,8 +487,7 @@ fa_status fa_align_iter(fa_ctx* c, void* K, float* log_u, float* log_v,
   ep.X = c->X;
   ep.rowmax_part = c->rowmax_part;
   // Z = W P2^T for P2 in {C2, A2bar^T}, cost assembly and log Gibbs kernel
-  FA_TRY(launch_spmm_right_cost(c->g2->d, n1, c->ld1, c->ld, c->intra2,
-                                c->g2->d.val_col, c->v_scale, c->Wt, ep, bf16, s));
+  FA_TRY(launch_spmm_right_cost(c->g2->d, n1, c->ld1, c->ld, c->recs2, c->Wt, ep, bf16, s));
   FA_TRY(launch_rowmax_reduce(n1, (int)(c->ld / 64), c->rowmax_part, c->rowmax, c->status, s));
   // row-stabilised kernel and the first column update a_1 (u = 1)
   const int Gn = normalize_groups(n1);

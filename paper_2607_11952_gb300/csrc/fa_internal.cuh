@@ -115,11 +115,9 @@ fa_status launch_spmm_pair_T(const DevGraph& g1, int n2, int64_t ldd, int64_t ld
                              cudaStream_t s);
 fa_status launch_spmm_T(const DevGraph& g, int n_cols, int64_t ldd, int64_t ldw, const void* recs,
                         const float* D, float* Wt, cudaStream_t s);
-fa_status launch_spmm_right_cost(const DevGraph& g2, int n1, int64_t ldw,
-                                 int64_t ldo, const float* qa, const float* qb,
-                                 const float* scale, const float* Wt,
-                                 const CostEpi& ep, bool k_bf16,
-                                 cudaStream_t s);
+fa_status launch_spmm_right_cost(const DevGraph& g2, int n1, int64_t ldw, int64_t ldo,
+                                 const void* recs, const float* Wt, const CostEpi& ep,
+                                 bool k_bf16, cudaStream_t s);
 fa_status launch_rowmax_reduce(int n1, int ntiles, const float* part,
                                float* rowmax, int* status, cudaStream_t s);
 fa_status launch_exp_vec(int n, const float* x, float* y, cudaStream_t s);

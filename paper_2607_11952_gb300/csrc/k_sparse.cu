@@ -16,8 +16,6 @@
 // (k_spmm): a gather engine with a transposed or a row-major store.
 #include <math.h>
 
-#include <stdlib.h>
-
 #include "fa_internal.cuh"
 #include "sweep_dev.cuh"
 
@@ -82,6 +80,10 @@ fa_status launch_edge_records(const DevGraph& g, const float* va, const float* v
   return FA_OK;
 }
 
+// A value every lane of the warp holds alike, in a form that the compiler
+// knows to be so: branches on it need no reconvergence code.
+__device__ __forceinline__ int uniform(int v) { return v; }
+
 __device__ __forceinline__ EdgeRec lds_edge(const EdgeRec* p) {
   const int4 v = *reinterpret_cast<const int4*>(p);
   return EdgeRec{v.x, v.y, __int_as_float(v.z), __int_as_float(v.w)};
@@ -92,7 +94,7 @@ __device__ __forceinline__ EdgeRec lds_edge(const EdgeRec* p) {
 // column panel of TJ = 32 V columns (V = 16 bytes of D per lane) and one
 // tile of TI rows of P per CTA.  OUT_T stores the product transposed, Wt[j,
 // i] (NV floats per element, TI consecutive i per column j); OUT_ROWS stores
-// alpha times it row-major.
+// alpha times it row-major, plus beta where seeds[j] = i.
 //
 // The tile's edges are one contiguous CSR range, split evenly over the NW
 // warps whatever the rows' degrees are: with one warp per row a hub row of
@@ -137,6 +139,34 @@ __device__ __forceinline__ uint4 ldg16(const char* p) {
   }
 }
 
+// A warp's edge records in 64 shared slots: the edge q steps before the
+// range's end in slot q & 63, refilled 32 at a time as they are used up.
+// Slots past the range hold its first edge, so that a gather running ahead
+// of the range's end reads a valid row.
+struct EdgeFeed {
+  const int4* last;     // the record of the range's last edge
+  int most;             // edges in the range - 1
+  int4 later;           // this lane's record of the batch after next
+  __device__ __forceinline__ EdgeFeed(const EdgeRec* recs, int ee, int cnt, EdgeRec* my, int lane)
+      : last(reinterpret_cast<const int4*>(recs) + (ee - 1)), most(cnt - 1) {
+    if (cnt > 0) {
+      *reinterpret_cast<int4*>(my + lane) = at(lane);
+      *reinterpret_cast<int4*>(my + 32 + lane) = at(32 + lane);
+      later = at(64 + lane);
+    }
+  }
+  __device__ __forceinline__ int4 at(int q) const { return __ldg(last - min(q, most)); }
+  // edges before q are done; q a multiple of the chunk
+  __device__ __forceinline__ void next(int q, EdgeRec* my, int lane) {
+    if ((q & 31) == 0) {
+      __syncwarp();
+      *reinterpret_cast<int4*>(my + ((q + 32 + lane) & 63)) = later;
+      later = at(q + 64 + lane);
+      __syncwarp();
+    }
+  }
+};
+
 template <typename TD, int NV, int TI, int NW>
 struct SpmmShape {
   static constexpr int V = 16 / (int)sizeof(TD);     // columns per lane
@@ -163,7 +193,7 @@ __global__ void __launch_bounds__(32 * NW, MINB) k_spmm(
   __shared__ int head_row[NW];
   const int i0 = blockIdx.x * TI;
   const int j0 = blockIdx.y * TJ;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
   unsigned char* mine = sm_raw + warp * Sh::kWarpBytes;
   for (int t = threadIdx.x; t <= TI; t += 32 * NW) rps[t] = rp[min(i0 + t, n)];
   int cur = -1, cnt, eb;
@@ -186,8 +216,8 @@ __global__ void __launch_bounds__(32 * NW, MINB) k_spmm(
   };
   {
     const int E0 = rp[i0], len = rp[min(i0 + TI, n)] - E0;
-    eb = E0 + (int)((int64_t)len * warp / NW);
-    const int ee = E0 + (int)((int64_t)len * (warp + 1) / NW);
+    eb = uniform(E0 + (int)((int64_t)len * warp / NW));
+    const int ee = uniform(E0 + (int)((int64_t)len * (warp + 1) / NW));
     cnt = ee - eb;
     // a lane past the operand's last column gathers the panel's first ones;
     // its results are never stored
@@ -195,21 +225,15 @@ __global__ void __launch_bounds__(32 * NW, MINB) k_spmm(
     const char* dcol = reinterpret_cast<const char*>(D + jl);
     const uint32_t ldb = (uint32_t)(ldd * (int64_t)sizeof(TD));
     EdgeRec* my = reinterpret_cast<EdgeRec*>(mine);   // edge ee - 1 - q in slot q & 63
-    const int4* rsrc = reinterpret_cast<const int4*>(recs) + (ee - 1 - lane);
-    int4 later;                                       // records of the batch after next
-    if (lane < cnt) *reinterpret_cast<int4*>(my + lane) = __ldg(rsrc);
-    if (32 + lane < cnt) *reinterpret_cast<int4*>(my + 32 + lane) = __ldg(rsrc - 32);
-    if (64 + lane < cnt) later = __ldg(rsrc - 64);
+    EdgeFeed feed(recs, ee, cnt, my, lane);
     __syncwarp();
     uint4 da[B], db[B];
-    // gathers of edges q .. q + B - 1; past the end the last edge's again
-    auto gather = [&](uint4 (&d)[B], int q) {
+    auto gather = [&](uint4 (&d)[B], const EdgeRec* p) {
 #pragma unroll
-      for (int u = 0; u < B; ++u)
-        d[u] = ldg16<A16>(dcol + (uint64_t)(uint32_t)my[min(q + u, cnt - 1) & 63].nb * ldb);
+      for (int u = 0; u < B; ++u) d[u] = ldg16<A16>(dcol + (uint64_t)(uint32_t)p[u].nb * ldb);
     };
-    auto add = [&](const uint4& d, int q) {
-      const EdgeRec er = lds_edge(my + (q & 63));
+    auto add = [&](const uint4& d, const EdgeRec* p) {
+      const EdgeRec er = lds_edge(p);
       if (er.row != cur) {
         if (cur >= 0) store_row(tile + (cur - i0) * RS);
         clear();
@@ -227,31 +251,28 @@ __global__ void __launch_bounds__(32 * NW, MINB) k_spmm(
       }
     };
     if (cnt > 0) {
-      gather(da, 0);
+      const EdgeRec* p = my;
+      gather(da, p);
       int q = 0;
       for (; q + 2 * B <= cnt; q += 2 * B) {
-        gather(db, q + B);
+        const EdgeRec* pn = my + ((q + 2 * B) & 63);
+        gather(db, p + B);
 #pragma unroll
-        for (int u = 0; u < B; ++u) add(da[u], q + u);
-        gather(da, q + 2 * B);
+        for (int u = 0; u < B; ++u) add(da[u], p + u);
+        gather(da, pn);
 #pragma unroll
-        for (int u = 0; u < B; ++u) add(db[u], q + B + u);
-        const int qn = q + 2 * B;
-        if ((qn & 31) == 0) {                         // a batch of 32 records is used up
-          __syncwarp();
-          if (qn + 32 + lane < cnt) *reinterpret_cast<int4*>(my + ((qn + 32 + lane) & 63)) = later;
-          if (qn + 64 + lane < cnt) later = __ldg(rsrc - (qn + 64));
-          __syncwarp();
-        }
+        for (int u = 0; u < B; ++u) add(db[u], p + B + u);
+        p = pn;
+        feed.next(q + 2 * B, my, lane);
       }
       if (q < cnt) {                                  // the last 1 .. 2 B - 1 edges
-        gather(db, q + B);
+        gather(db, p + B);
 #pragma unroll
         for (int u = 0; u < B; ++u)
-          if (q + u < cnt) add(da[u], q + u);
+          if (q + u < cnt) add(da[u], p + u);
 #pragma unroll
         for (int u = 0; u < B; ++u)
-          if (q + B + u < cnt) add(db[u], q + B + u);
+          if (q + B + u < cnt) add(db[u], p + B + u);
       }
     }
   }
@@ -442,220 +463,269 @@ fa_status launch_spmm_T(const DevGraph& g, int n_cols, int64_t ldd, int64_t ldw,
 }
 
 // ------------------------------------------------------------ right SpMM with cost
-// Largest t in [0, n) with p[t] <= e, for p[0] <= e < p[n] (p nondecreasing).
-template <int N>
-__device__ __forceinline__ int seg_of(const int* p, int e) {
-  int lo = 0, hi = N;
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (p[mid] <= e) lo = mid; else hi = mid;
-  }
-  return lo;
-}
-
 // Cost assembly + log Gibbs kernel (Phase 2 of Algorithm 1, Eq. 2, proximal step):
 //   C   = C_node + lam_e Z_e - lam_n log max(Z_n, delta) + lam_a C_anc
 //   x   = -C/eps + (lam_p/eps) (log u_i + log K_prev_ij + log v_j)
-// stored as float32, plus the per-(row, 64-column tile) maximum of x.
+// stored as float32, plus the per-(row, 64-column tile) maximum of x, with
+// Z[i, j] = sum_l P2[j, l] s_l W^T[l, i] for both value sets (recs: P2's
+// records, W^T pairs interleaved).
 __device__ __forceinline__ float to_f32(float v) { return v; }
 __device__ __forceinline__ float to_f32(__nv_bfloat16 v) { return __bfloat162float(v); }
 
-// CTA tile: 64 columns j x 64 rows i.  The tile's neighbour lists are one
-// contiguous CSR range [rp[j0], rp[j0+64]); it is split evenly over the 8
-// warps by edge count (not by column), so a hub column's gathers are shared
-// and the warps of a CTA finish together.  A warp loads 32 edges at a time
-// lane-parallel (column index, both weights times the scaling s_l, and the
-// output column found by binary search in the tile's row pointers), then
-// broadcasts them and keeps GU gathers of W^T[l, i0:i0+64] (one float4 per
-// lane: rows 2 lane, 2 lane + 1, both value sets) in flight.  The sums are
-// formed without atomics, in a fixed order: a column whose edges lie
-// wholly in one warp's range is stored into the shared tile by that warp;
-// a column split between warps (at most the first and the last column of a
-// warp's range) leaves one partial per warp in that warp's head or tail
-// slot, and the epilogue adds a split column's partials in warp order.  The
-// epilogue walks rows, lanes over columns, so the C_node, K_prev and X rows
-// are coalesced.  Shared tiles are XOR-swizzled by row so both the stores
-// (lanes over rows) and the epilogue (lanes over columns) are free of bank
-// conflicts up to 2 ways.  Two runs give bit-identical results.
+// Natural logarithm of 0 <= x < infinity for the log-kernel: x = 2^e m with m
+// in [0.75, 1.5), log x = e ln 2 + ln 2 lg2(m).  The hardware's lg2 is within
+// 2^-22 absolutely on (0.5, 2), 1.7e-7 in natural units, below the rounding
+// of a result of more than 2 (1.2e-7 to 4e-6 at the |log| of 2 to 90 met
+// here); lg2(1) = 0 exactly, denormals are scaled by 2^23 first, 0 gives
+// -infinity.  The epilogue takes two logarithms per element, and logf was
+// most of its instructions.
+__device__ __forceinline__ float log_pos(float x) {
+  const bool tiny = x < 1.17549435e-38f;
+  const uint32_t b = __float_as_uint(tiny ? x * 8388608.f : x);
+  const int e = (int)(b - 0x3f400000u) >> 23;
+  const float m = __uint_as_float(b - ((uint32_t)e << 23));
+  float l;
+  asm("lg2.approx.f32 %0, %1;" : "=f"(l) : "f"(m));
+  const float r = fmaf((float)(tiny ? e - 23 : e), 0.693147180559945f, l * 0.693147180559945f);
+  return x == 0.f ? -INFINITY : r;
+}
+// negative numbers, infinities and NaN: out of line, never in a valid plan
+__device__ __noinline__ float log_any(float x) { return logf(x); }
+
+template <bool VEC>
+__device__ __forceinline__ float2 load_pair(const float* p) {
+  if constexpr (VEC) return __ldcs(reinterpret_cast<const float2*>(p));
+  return make_float2(p[0], p[1]);
+}
+__device__ __forceinline__ float2 load_kernel_pair(const float* p) {
+  return __ldcs(reinterpret_cast<const float2*>(p));
+}
+__device__ __forceinline__ float2 load_kernel_pair(const __nv_bfloat16* p) {
+  const uint32_t u = __ldcs(reinterpret_cast<const uint32_t*>(p));
+  return make_float2(__uint_as_float(u << 16), __uint_as_float(u & 0xffff0000u));
+}
+
+// CTA tile: 64 columns j x 64 rows i.  The gathers are the engine's of
+// k_spmm with the roles of rows and columns exchanged: the tile's columns'
+// edges split evenly over the 8 warps, walked from the last to the first in
+// two batches of gathers, a column split between warps parked and added in
+// warp order (no atomics: two runs give identical bits).  A lane holds rows
+// 2 lane and 2 lane + 1 as (e, n) pairs, so one paired FMA adds both value
+// sets of a row with the record's weight pair.  The epilogue walks rows, a
+// lane's columns 2 lane and 2 lane + 1, four rows at a time; their four
+// maxima are reduced together (6 shuffles instead of 20).  The shared
+// tile is column-major, columns 130 floats apart: 2-way conflicts both ways.
+//
+// What bounds it: 512-byte gathers of W^T from L2 (8 nnz2 n1 bytes) and the
+// issue slots of the epilogue (two logarithms per element); HBM moves
+// (16 + b) n1 n2 bytes.  Measured on GB300, 50,000 nodes of degree 10, BF16:
+// 28.9 -> 18.1 ms (200 GB of gathers, 45 GB of HBM); 10,000 nodes FP32: 1.07
+// -> 0.67 ms.  Without its edges the kernel takes 0.3 ms at 10,000 nodes.
+// 5 CTAs per SM with batches of 2 (48 registers): 20.8 ms; a scan of the
+// row's anchors per element instead of the tile's flag: 19.8 ms.
 constexpr int kRT = 64;    // rows per tile
 constexpr int kCT = 64;    // columns per tile
+constexpr int kZS = 2 * kRT + 2;   // floats between columns of the shared tile
 
-__device__ __forceinline__ int sw_idx(int r, int c) { return r * kCT + (c ^ (r & 31)); }
-
-template <typename TK, int MINB, int GU>
-__global__ void __launch_bounds__(256, MINB) k_spmm_right_cost(
+template <typename TK, bool VEC>
+__global__ void __launch_bounds__(256, 4) k_spmm_right_cost(
     int n1, int n2, int64_t ldw, int64_t ldo, const int32_t* __restrict__ rp,
-    const int32_t* __restrict__ ci, const float* __restrict__ qa,
-    const float* __restrict__ qb, const float* __restrict__ scale,
-    const float* __restrict__ Wt, CostEpi ep) {
-  __shared__ float ze_s[kRT * kCT];
-  __shared__ float zn_s[kRT * kCT];
-  __shared__ __align__(16) float4 split_s[8][2][kRT / 2];   // [warp][head/tail][lane]: a0 b0 a1 b1
-  __shared__ int split_col[8][2];                            // column of each slot, -1 if unused
-  __shared__ __align__(16) EdgeRec edges[8][32];
-  __shared__ int rps[kCT + 1];
+    const EdgeRec* __restrict__ recs, const float* __restrict__ Wt, CostEpi ep) {
+  constexpr int B = 4;                                // gathers per batch
+  __shared__ __align__(16) float z[kCT * kZS];        // [column][row](e, n)
+  __shared__ __align__(16) EdgeRec edges[8][64];      // records; then a parked column
+  __shared__ int rps[kCT + 1], head_col[8], any_part[2];
+  __shared__ uint32_t anc[kRT][2];                    // anchors of a row: bit per column
+  __shared__ float lus[kRT];
   const int j0 = blockIdx.x * kCT, i0 = blockIdx.y * kRT;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int t = threadIdx.x; t < kRT * kCT; t += blockDim.x) {
-    ze_s[t] = 0.f;
-    zn_s[t] = 0.f;
-  }
+  const int warp = uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (threadIdx.x <= kCT) rps[threadIdx.x] = rp[min(j0 + (int)threadIdx.x, n2)];
-  if (threadIdx.x < 16) split_col[threadIdx.x >> 1][threadIdx.x & 1] = -1;
-  __syncthreads();
-
-  // ---- gathers: Z_e[i, j] and Z_n[i, j] for rows 2 lane, 2 lane + 1
-  {
-    const int E0 = rps[0], len = rps[kCT] - E0;
-    const int eb = E0 + (int)((int64_t)len * warp / 8);
-    const int ee = E0 + (int)((int64_t)len * (warp + 1) / 8);
-    const int r0 = 2 * lane, r1 = 2 * lane + 1;
-    const float* wbase = Wt + (int64_t)(i0 + r0) * 2;
-    int cur = -1;
-    float a0 = 0.f, b0 = 0.f, a1 = 0.f, b1 = 0.f;
-    auto flush = [&]() {
-      if (cur >= 0) {
-        const bool starts_before = rps[cur] < eb, ends_after = rps[cur + 1] > ee;
-        if (!starts_before && !ends_after) {   // the whole column is this warp's
-          ze_s[sw_idx(r0, cur)] = a0;
-          zn_s[sw_idx(r0, cur)] = b0;
-          ze_s[sw_idx(r1, cur)] = a1;
-          zn_s[sw_idx(r1, cur)] = b1;
-        } else {                               // split: head (first) or tail slot
-          const int slot = starts_before ? 0 : 1;
-          split_s[warp][slot][lane] = make_float4(a0, b0, a1, b1);
-          if (lane == 0) split_col[warp][slot] = cur;
-        }
+  if (threadIdx.x >= 128 && threadIdx.x < 128 + kRT) {
+    // few tiles hold an anchor at all: one flag per tile, a bit per column
+    const int r = threadIdx.x - 128, i = i0 + r;
+    uint32_t m[2] = {0u, 0u};
+    if (i < n1)
+      for (int a = ep.anc_ptr[i], a1 = ep.anc_ptr[i + 1]; a < a1; ++a) {
+        const int d = ep.anc_col[a] - j0;
+        if (d >= 0 && d < kCT) m[d >> 5] |= 1u << (d & 31);
       }
-      a0 = b0 = a1 = b1 = 0.f;
+    anc[r][0] = m[0];
+    anc[r][1] = m[1];
+    lus[r] = ep.log_u[min(i, n1 - 1)];
+    const bool any = __any_sync(0xffffffffu, (m[0] | m[1]) != 0u);
+    if ((threadIdx.x & 31) == 0) any_part[(threadIdx.x >> 5) & 1] = any;
+  }
+  int cur = -1, cnt, eb;
+  float a0 = 0.f, b0 = 0.f, a1 = 0.f, b1 = 0.f;       // (e, n) of rows 2 lane, 2 lane + 1
+  auto store_col = [&](float* dst) {
+    *reinterpret_cast<float2*>(dst + 4 * lane) = make_float2(a0, b0);
+    *reinterpret_cast<float2*>(dst + 4 * lane + 2) = make_float2(a1, b1);
+  };
+  {
+    const int E0 = rp[min(j0, n2)], len = rp[min(j0 + kCT, n2)] - E0;
+    eb = uniform(E0 + (int)((int64_t)len * warp / 8));
+    const int ee = uniform(E0 + (int)((int64_t)len * (warp + 1) / 8));
+    cnt = ee - eb;
+    const char* wrow = reinterpret_cast<const char*>(Wt + (int64_t)(i0 + 2 * lane) * 2);
+    const uint32_t ldb = (uint32_t)(ldw * 8);
+    EdgeRec* my = edges[warp];                        // edge ee - 1 - q in slot q & 63
+    EdgeFeed feed(recs, ee, cnt, my, lane);
+    __syncwarp();
+    uint4 da[B], db[B];
+    auto gather = [&](uint4 (&d)[B], const EdgeRec* p) {
+#pragma unroll
+      for (int u = 0; u < B; ++u) d[u] = ldg16<true>(wrow + (uint64_t)(uint32_t)p[u].nb * ldb);
     };
-    EdgeRec* my = edges[warp];
-    for (int base = eb; base < ee; base += 32) {
-      const int e = base + lane;
-      if (e < ee) {
-        const int l = ci[e];
-        const float sl = scale ? scale[l] : 1.f;
-        my[lane] = EdgeRec{l, seg_of<kCT>(rps, e), qa[e] * sl, qb[e] * sl};
+    auto add = [&](const uint4& d, const EdgeRec* p) {
+      const int4 er = *reinterpret_cast<const int4*>(p);
+      if (er.y != cur) {
+        if (cur >= 0) store_col(z + (cur - j0) * kZS);
+        a0 = b0 = a1 = b1 = 0.f;
+        cur = er.y;
       }
-      __syncwarp();
-      const int cnt = min(32, ee - base);
-      for (int u = 0; u < cnt; u += GU) {
-        float4 w[GU];
+      const float wa = __int_as_float(er.z), wb = __int_as_float(er.w);
+      a0 = fmaf(wa, __uint_as_float(d.x), a0);
+      b0 = fmaf(wb, __uint_as_float(d.y), b0);
+      a1 = fmaf(wa, __uint_as_float(d.z), a1);
+      b1 = fmaf(wb, __uint_as_float(d.w), b1);
+    };
+    if (cnt > 0) {
+      const EdgeRec* p = my;
+      gather(da, p);
+      int q = 0;
+      for (; q + 2 * B <= cnt; q += 2 * B) {
+        const EdgeRec* pn = my + ((q + 2 * B) & 63);
+        gather(db, p + B);
 #pragma unroll
-        for (int k = 0; k < GU; ++k)
-          if (u + k < cnt)
-            w[k] = __ldg(reinterpret_cast<const float4*>(wbase + (int64_t)my[u + k].nb * ldw * 2));
+        for (int u = 0; u < B; ++u) add(da[u], p + u);
+        gather(da, pn);
 #pragma unroll
-        for (int k = 0; k < GU; ++k) {
-          if (u + k < cnt) {
-            const EdgeRec er = lds_edge(&my[u + k]);
-            if (er.row != cur) {
-              flush();
-              cur = er.row;
-            }
-            a0 = fmaf(er.wa, w[k].x, a0);
-            b0 = fmaf(er.wb, w[k].y, b0);
-            a1 = fmaf(er.wa, w[k].z, a1);
-            b1 = fmaf(er.wb, w[k].w, b1);
-          }
-        }
+        for (int u = 0; u < B; ++u) add(db[u], p + B + u);
+        p = pn;
+        feed.next(q + 2 * B, my, lane);
       }
-      __syncwarp();
+      if (q < cnt) {
+        gather(db, p + B);
+#pragma unroll
+        for (int u = 0; u < B; ++u)
+          if (q + u < cnt) add(da[u], p + u);
+#pragma unroll
+        for (int u = 0; u < B; ++u)
+          if (q + B + u < cnt) add(db[u], p + B + u);
+      }
     }
-    flush();
   }
   __syncthreads();
-  // ---- split columns: the warps' partials in warp order (head before
-  // tail within a warp: a warp's head column precedes its tail column)
   {
-    if (threadIdx.x < kRT) {
-      const int row = threadIdx.x, ln = row >> 1, hi = row & 1;
-      int col = -1;
-      float za = 0.f, zb = 0.f;
-      for (int w = 0; w < 8; ++w) {
+    const bool parked = cnt > 0 && rps[cur - j0] < eb;   // begun in an earlier warp's range
+    if (cnt > 0)
+      store_col(parked ? reinterpret_cast<float*>(edges[warp]) : z + (cur - j0) * kZS);
+    if (lane == 0) head_col[warp] = parked ? cur - j0 : -1;
+  }
+  __syncthreads();
+  if (threadIdx.x < 2 * kRT) {
 #pragma unroll
-        for (int sl = 0; sl < 2; ++sl) {
-          const int c = split_col[w][sl];
-          if (c < 0) continue;
-          if (c != col) {
-            if (col >= 0) {
-              ze_s[sw_idx(row, col)] = za;
-              zn_s[sw_idx(row, col)] = zb;
-            }
-            col = c;
-            za = zb = 0.f;
-          }
-          const float4 v = split_s[w][sl][ln];
-          za += hi ? v.z : v.x;
-          zb += hi ? v.w : v.y;
-        }
-      }
-      if (col >= 0) {
-        ze_s[sw_idx(row, col)] = za;
-        zn_s[sw_idx(row, col)] = zb;
-      }
+    for (int w = 1; w < 8; ++w) {
+      const int c = head_col[w];
+      if (c >= 0) z[c * kZS + threadIdx.x] += reinterpret_cast<const float*>(edges[w])[threadIdx.x];
     }
   }
   __syncthreads();
 
-  // ---- epilogue: rows over warps, columns j0 + lane and j0 + 32 + lane
+  // ---- epilogue: 8 rows per warp, four at a time
   const float inv_eps = 1.0f / ep.eps;
   const float prox = ep.lam_p * inv_eps;
   const float c_off = -logf(ep.eps_anc);          // C_anc off the anchors
   const float c_on = -logf(ep.eps_anc + 1.0f);    // C_anc on an anchor
   const TK* Kp = static_cast<const TK*>(ep.K_prev);
-  for (int r = warp; r < kRT; r += 8) {
-    const int i = i0 + r;
-    if (i >= n1) break;
-    const float lu = ep.log_u[i];
-    const int a0 = ep.anc_ptr[i], a1 = ep.anc_ptr[i + 1];
-    const int64_t row = (int64_t)i * ldo;
-    float mx = -INFINITY;
+  const int c = 2 * lane, j = j0 + c;
+  const bool in0 = j < n2, in1 = j + 1 < n2;
+  const bool any0 = in0 && rps[c + 1] > rps[c], any1 = in1 && rps[c + 2] > rps[c + 1];
+  const float lv0 = in0 ? ep.log_v[j] : 0.f, lv1 = in1 ? ep.log_v[j + 1] : 0.f;
+  const float* z0 = z + c * kZS;
+  const bool any_anchor = any_part[0] | any_part[1];
+  // 32-bit offsets within the tile
+  const int64_t tile0 = (int64_t)i0 * ldo + j;
+  const float* Ct = ep.C_node + tile0;
+  const TK* Kt = Kp + tile0;
+  float* Xt = ep.X + tile0;
+  const uint32_t ldo32 = (uint32_t)ldo;
+  const int rlast = n1 - 1 - i0;                   // the last row, within the tile
+#pragma unroll 1
+  for (int r0 = warp * 8; r0 < warp * 8 + 8; r0 += 4) {
+    float mx[4];
+    float2 cn[4], kp[4];
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int c = lane + 32 * h, j = j0 + c;
-      float x = -INFINITY;
-      if (j < n2) {
-        const int si = sw_idx(r, c);
-        float canc = c_off;
-        for (int a = a0; a < a1; ++a)
-          if (ep.anc_col[a] == j) canc = c_on;
-        const float C = ep.C_node[row + j] + ep.lam_e * ze_s[si] -
-                        ep.lam_n * logf(fmaxf(zn_s[si], ep.delta)) + ep.lam_a * canc;
-        x = -C * inv_eps;
-        if (prox != 0.f) x += prox * (lu + logf(to_f32(Kp[row + j])) + ep.log_v[j]);
-        mx = fmaxf(mx, x);
-      }
-      ep.X[row + j] = x;
+    for (int t = 0; t < 4; ++t) {                  // rows past n1 read the last row again
+      const uint32_t at = (uint32_t)min(r0 + t, rlast) * ldo32;
+      cn[t] = load_pair<VEC>(Ct + at);
+      kp[t] = prox != 0.f ? load_kernel_pair(Kt + at) : make_float2(1.f, 1.f);
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if (lane == 0) ep.rowmax_part[(int64_t)blockIdx.x * n1 + i] = mx;
+    for (int t = 0; t < 4; ++t) {
+      const int r = r0 + t;
+      mx[t] = -INFINITY;
+      if (r <= rlast) {                            // warp-uniform
+        const float2 za = any0 ? *reinterpret_cast<const float2*>(z0 + 2 * r) : make_float2(0.f, 0.f);
+        const float2 zb = any1 ? *reinterpret_cast<const float2*>(z0 + kZS + 2 * r) : make_float2(0.f, 0.f);
+        const float lu = lus[r];
+        float can0 = c_off, can1 = c_off;
+        if (any_anchor) {
+          const uint32_t m = anc[r][c >> 5] >> (c & 31);
+          if (m & 1u) can0 = c_on;
+          if (m & 2u) can1 = c_on;
+        }
+        const float n0 = fmaxf(za.y, ep.delta), n1v = fmaxf(zb.y, ep.delta);
+        float ln0 = log_pos(n0), ln1 = log_pos(n1v), lk0 = log_pos(kp[t].x), lk1 = log_pos(kp[t].y);
+        if ((__float_as_uint(n0) | __float_as_uint(n1v) | __float_as_uint(kp[t].x) |
+             __float_as_uint(kp[t].y)) >= 0x7f800000u) {
+          ln0 = log_any(n0);
+          ln1 = log_any(n1v);
+          lk0 = log_any(kp[t].x);
+          lk1 = log_any(kp[t].y);
+        }
+        const float C0 = cn[t].x + ep.lam_e * za.x - ep.lam_n * ln0 + ep.lam_a * can0;
+        const float C1 = cn[t].y + ep.lam_e * zb.x - ep.lam_n * ln1 + ep.lam_a * can1;
+        float x0 = -C0 * inv_eps, x1 = -C1 * inv_eps;
+        if (prox != 0.f) {
+          x0 += prox * (lu + lk0 + lv0);
+          x1 += prox * (lu + lk1 + lv1);
+        }
+        if (!in0) x0 = -INFINITY;                  // padding columns
+        if (!in1) x1 = -INFINITY;
+        __stcs(reinterpret_cast<float2*>(Xt + (uint32_t)r * ldo32), make_float2(x0, x1));
+        mx[t] = fmaxf(x0, x1);
+      }
+    }
+    // four rows' maxima: lanes 0-7 end with row r0's, 8-15 r0 + 1's, ...
+    {
+      const bool hi = lane & 16;
+      const float h0 = hi ? mx[2] : mx[0], h1 = hi ? mx[3] : mx[1];
+      const float s0 = hi ? mx[0] : mx[2], s1 = hi ? mx[1] : mx[3];
+      const float g0 = fmaxf(h0, __shfl_xor_sync(0xffffffffu, s0, 16));
+      const float g1 = fmaxf(h1, __shfl_xor_sync(0xffffffffu, s1, 16));
+      const bool lo = lane & 8;
+      float m = fmaxf(lo ? g1 : g0, __shfl_xor_sync(0xffffffffu, lo ? g0 : g1, 8));
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+      const int i = i0 + r0 + (lane >> 3);
+      if ((lane & 7) == 0 && i < n1) ep.rowmax_part[(int64_t)blockIdx.x * n1 + i] = m;
+    }
   }
 }
 
-fa_status launch_spmm_right_cost(const DevGraph& g2, int n1, int64_t ldw,
-                                 int64_t ldo, const float* qa, const float* qb,
-                                 const float* scale, const float* Wt,
-                                 const CostEpi& ep, bool k_bf16,
-                                 cudaStream_t s) {
-  // resident CTAs per SM the register budget is sized for: 3 (80 registers)
-  // measured faster than 2 (88) on GB300 at 10k and 50k
-  // Resident CTAs per SM the register budget is sized for, and gathers in
-  // flight per warp.  Measured on GB300 (one outer iteration, 50k BF16):
-  // 5 CTAs x 4 gathers (48 registers; 5 x 45 KB of shared memory fit the
-  // SM) 46.1 ms, 4 x 6 48.8 ms, 3 x 8 56.1 ms, 2 x 16 72.3 ms: the gathers'
-  // latency is hidden by more warps, not by deeper warps.  FA_PASSB_MINB=4
-  // or 3 selects those shapes (tuning).
-  const char* mb = getenv("FA_PASSB_MINB");
-  const int minb = (mb && atoi(mb) == 3) ? 3 : (mb && atoi(mb) == 4) ? 4 : 5;
+fa_status launch_spmm_right_cost(const DevGraph& g2, int n1, int64_t ldw, int64_t ldo,
+                                 const void* recs, const float* Wt, const CostEpi& ep,
+                                 bool k_bf16, cudaStream_t s) {
   dim3 grid((unsigned)(ldo / kCT), (unsigned)((n1 + kRT - 1) / kRT));
-#define FA_PB(T, M, GU) \
-  k_spmm_right_cost<T, M, GU><<<grid, 256, 0, s>>>(n1, g2.n, ldw, ldo, g2.row_ptr, g2.col, qa, qb, scale, Wt, ep)
+  const EdgeRec* rec = static_cast<const EdgeRec*>(recs);
+  const bool vec = (reinterpret_cast<uintptr_t>(ep.C_node) & 7u) == 0;
+#define FA_PB(T, VEC) \
+  k_spmm_right_cost<T, VEC><<<grid, 256, 0, s>>>(n1, g2.n, ldw, ldo, g2.row_ptr, rec, Wt, ep)
   if (k_bf16) {
-    if (minb == 4) FA_PB(__nv_bfloat16, 4, 6); else if (minb == 5) FA_PB(__nv_bfloat16, 5, 4); else FA_PB(__nv_bfloat16, 3, 8);
+    if (vec) FA_PB(__nv_bfloat16, true); else FA_PB(__nv_bfloat16, false);
   } else {
-    if (minb == 4) FA_PB(float, 4, 6); else if (minb == 5) FA_PB(float, 5, 4); else FA_PB(float, 3, 8);
+    if (vec) FA_PB(float, true); else FA_PB(float, false);
   }
 #undef FA_PB
   FA_LAUNCHED("k_spmm_right_cost");
