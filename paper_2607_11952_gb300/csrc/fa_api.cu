@@ -335,7 +335,8 @@ fa_status fa_node_cost(fa_ctx* c, const float* X1, const float* X2, int32_t d,
   const int n1 = c->n1, n2 = c->n2;
   const int L = n_anchor;
   // anchors: host checks, per-graph node lists and the row-sorted list
-  std::vector<int32_t> a1(std::max(L, 1)), a2(std::max(L, 1));
+  const int64_t ldr = round_up(std::max(L, 1), 64);
+  std::vector<int32_t> a1(ldr, -1), a2(ldr, -1);   // -1: a padding column of R
   std::vector<std::pair<int32_t, int32_t>> byrow(L);
   for (int l = 0; l < L; ++l) {
     const int32_t i = anchors[2 * l], j = anchors[2 * l + 1];
@@ -361,7 +362,6 @@ fa_status fa_node_cost(fa_ctx* c, const float* X1, const float* X2, int32_t d,
   FA_CUDA(cudaMemcpyAsync(c->anc_col, acol.data(), std::max(L, 1) * sizeof(int32_t), cudaMemcpyHostToDevice, s));
   c->n_anchor = L;
 
-  const int64_t ldr = round_up(std::max(L, 1), 64);
   const int64_t ldx = round_up(std::max(d, 1), 64);
   float *R1a = nullptr, *R1b = nullptr, *R2a = nullptr, *R2b = nullptr;
   float *X1h = nullptr, *X2h = nullptr;
@@ -393,10 +393,10 @@ fa_status fa_node_cost(fa_ctx* c, const float* X1, const float* X2, int32_t d,
   FA_STEP(amalloc((void**)&R2b, (size_t)n2 * ldr * 4));
   FA_STEP(amalloc((void**)&X1h, (size_t)n1 * ldx * 4));
   FA_STEP(amalloc((void**)&X2h, (size_t)n2 * ldx * 4));
-  FA_STEP(amalloc((void**)&da1, (size_t)std::max(L, 1) * 4));
-  FA_STEP(amalloc((void**)&da2, (size_t)std::max(L, 1) * 4));
-  if (cudaMemcpyAsync(da1, a1.data(), std::max(L, 1) * 4, cudaMemcpyHostToDevice, s) != cudaSuccess ||
-      cudaMemcpyAsync(da2, a2.data(), std::max(L, 1) * 4, cudaMemcpyHostToDevice, s) != cudaSuccess) {
+  FA_STEP(amalloc((void**)&da1, (size_t)ldr * 4));
+  FA_STEP(amalloc((void**)&da2, (size_t)ldr * 4));
+  if (cudaMemcpyAsync(da1, a1.data(), ldr * 4, cudaMemcpyHostToDevice, s) != cudaSuccess ||
+      cudaMemcpyAsync(da2, a2.data(), ldr * 4, cudaMemcpyHostToDevice, s) != cudaSuccess) {
     set_error("fa_node_cost: anchor upload failed");
     freeall();
     return FA_ERR_CUDA;
@@ -408,16 +408,14 @@ fa_status fa_node_cost(fa_ctx* c, const float* X1, const float* X2, int32_t d,
   FA_STEP(launch_onehot(n1, L, ldr, da1, R1a, s));
   FA_STEP(launch_onehot(n2, L, ldr, da2, R2a, s));
   for (int t = 0; t < c->p.k_rwr; ++t) {
-    FA_STEP(launch_rwr_step(c->g1->d, ldr, beta, c->recs1, R1a, R1b, s));
-    FA_STEP(launch_add_onehot(L, ldr, da1, beta, R1b, s));
+    FA_STEP(launch_rwr_step(c->g1->d, ldr, beta, c->recs1, da1, R1a, R1b, s));
     std::swap(R1a, R1b);
-    FA_STEP(launch_rwr_step(c->g2->d, ldr, beta, c->recs2, R2a, R2b, s));
-    FA_STEP(launch_add_onehot(L, ldr, da2, beta, R2b, s));
+    FA_STEP(launch_rwr_step(c->g2->d, ldr, beta, c->recs2, da2, R2a, R2b, s));
     std::swap(R2a, R2b);
   }
   // Algorithm 1, intra-graph costs: SDDMM for C1 (1/deg i) and C2 (1/deg l)
-  FA_STEP(launch_sddmm(c->g1->d, L, ldr, R1a, false, c->intra1, s));
-  FA_STEP(launch_sddmm(c->g2->d, L, ldr, R2a, true, c->intra2, s));
+  FA_STEP(launch_sddmm(c->g1->d, ldr, R1a, false, c->intra1, s));
+  FA_STEP(launch_sddmm(c->g2->d, ldr, R2a, true, c->intra2, s));
   // attributes
   if (d > 0) {
     FA_STEP(launch_normalize_rows(n1, d, X1, ldx, c->p.normalize_features != 0, X1h, s));

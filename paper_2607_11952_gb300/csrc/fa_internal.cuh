@@ -73,13 +73,11 @@ constexpr size_t kEdgeRecBytes = 16;      // one stored entry's record
 fa_status launch_edge_records(const DevGraph& g, const float* va, const float* vb,
                               const float* log_scale, void* recs, cudaStream_t s);
 fa_status launch_rwr_step(const DevGraph& g, int64_t ldr, float beta, const void* recs,
-                          const float* Rin, float* Rout, cudaStream_t s);
-fa_status launch_add_onehot(int L, int64_t ldr, const int32_t* nodes,
-                            float value, float* R, cudaStream_t s);
+                          const int32_t* seeds, const float* Rin, float* Rout, cudaStream_t s);
 fa_status launch_onehot(int n, int L, int64_t ldr, const int32_t* nodes,
                         float* R, cudaStream_t s);
-fa_status launch_sddmm(const DevGraph& g, int L, int64_t ldr, const float* R,
-                       bool weight_by_col, float* out, cudaStream_t s);
+fa_status launch_sddmm(const DevGraph& g, int64_t ldr, const float* R, bool weight_by_col,
+                       float* out, cudaStream_t s);
 fa_status launch_normalize_rows(int n, int d, const float* X, int64_t ldx,
                                 bool normalize, float* Xh, cudaStream_t s);
 fa_status launch_node_cost_simt(int n1, int n2, int L, int64_t ldr,
