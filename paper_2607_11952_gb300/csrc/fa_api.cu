@@ -5,6 +5,7 @@
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
+#include <cstdlib>
 #include <cstring>
 #include <vector>
 
@@ -228,7 +229,7 @@ fa_status fa_ctx_destroy(fa_ctx* c) {
   dfree(c->colpart); dfree(c->u_scale); dfree(c->v_scale);
   dfree(c->logv_buf[0]); dfree(c->logv_buf[1]);
   dfree(c->intra1); dfree(c->intra2); dfree(c->anc_ptr); dfree(c->anc_col);
-  dfree(c->err_part); dfree(c->ticket); dfree(c->err); dfree(c->status);
+  dfree(c->err_part); dfree(c->ticket); dfree(c->result); dfree(c->small_words);
   dfree(c->diff);
   for (auto& ev : c->sweep_events) cudaEventDestroy(ev);
   delete c;
@@ -268,6 +269,7 @@ fa_status fa_ctx_create(const fa_graph* g1, const fa_graph* g2,
   SweepPlan sp = plan_sweep(c->n1, c->ld, bf16, 1 << 20);
   int maxact = sp.Q >= 1 ? sweep_max_active_clusters(sp, bf16) : 0;
   c->G_sweep = std::max(1, maxact);
+  c->small_C = solve_small_clusters(c->n1, c->ld, bf16);
   c->maxG = std::max(c->G_sweep, normalize_groups(c->n1));
   const int64_t n1 = c->n1, n2 = c->n2, ld = c->ld, ld1 = c->ld1;
   fa_status st;
@@ -289,14 +291,17 @@ fa_status fa_ctx_create(const fa_graph* g1, const fa_graph* g2,
       (st = dalloc(&c->anc_col, 1, acc)) != FA_OK ||
       (st = dalloc(&c->err_part, (size_t)col_finalize_max_blocks((int)n2), acc)) != FA_OK ||
       (st = dalloc(&c->ticket, 1, acc)) != FA_OK ||
-      (st = dalloc(&c->err, 1, acc)) != FA_OK ||
-      (st = dalloc(&c->diff, (size_t)kPlanDiffBlocks + 1, acc)) != FA_OK ||
-      (st = dalloc(&c->status, 1, acc)) != FA_OK) {
+      (st = dalloc(&c->result, 1, acc)) != FA_OK ||
+      (st = dalloc(&c->small_words, solve_small_words(c->small_C, c->ld), acc)) != FA_OK ||
+      (st = dalloc(&c->diff, (size_t)kPlanDiffBlocks + 1, acc)) != FA_OK) {
     fa_ctx_destroy(c);
     return st;
   }
+  c->err = &c->result->err;
+  c->status = &c->result->status;
   if (cudaMemset(c->ticket, 0, sizeof(unsigned)) != cudaSuccess ||
-      cudaMemset(c->status, 0, sizeof(int)) != cudaSuccess ||
+      cudaMemset(c->result, 0, sizeof(SolveResult)) != cudaSuccess ||
+      (c->small_C > 0 && cudaMemset(c->small_words, 0, solve_small_words(c->small_C, c->ld)) != cudaSuccess) ||
       cudaMemset(c->anc_ptr, 0, (n1 + 1) * sizeof(int32_t)) != cudaSuccess ||
       cudaMemset(c->intra1, 0, std::max<int64_t>(1, g1->d.nnz) * sizeof(float)) != cudaSuccess ||
       cudaMemset(c->intra2, 0, std::max<int64_t>(1, g2->d.nnz) * sizeof(float)) != cudaSuccess) {
@@ -497,6 +502,47 @@ fa_status fa_align_iter(fa_ctx* c, void* K, float* log_u, float* log_v,
 }
 
 // ------------------------------------------------------------ Phase 3
+// The sweep's tuning switches ask for the sweep itself, as does its timing.
+static bool sweep_forced(const fa_ctx* c) {
+  static const char* const kNames[] = {"FA_SWEEP_KIND", "FA_SWEEP_Q", "FA_SWEEP_R", "FA_SWEEP_NS",
+                                       "FA_SWEEP_NT", "FA_SWEEP_G", "FA_SWEEP_SMAX",
+                                       "FA_SWEEP_ANYQ", "FA_SWEEP_L", "FA_SWEEP_MB"};
+  if (c->timing) return true;
+  for (const char* n : kNames) {
+    const char* v = getenv(n);
+    if (v && *v) return true;
+  }
+  return false;
+}
+
+// Reads back what a solve reports (the stream is synchronised) and turns it
+// into the call's results.  it: iterations done, 0 for a one-launch solve,
+// which counts them itself.
+static fa_status finish_solve(fa_ctx* c, int it, double tol, int32_t* iters_out, double* err_out,
+                              cudaStream_t s) {
+  FA_CUDA(cudaMemcpyAsync(&c->host_result, c->result, sizeof(SolveResult), cudaMemcpyDeviceToHost, s));
+  FA_CUDA(cudaStreamSynchronize(s));
+  const SolveResult r = c->host_result;
+  if (it == 0) it = r.iters;
+  if (r.status != 0) FA_CUDA(cudaMemsetAsync(c->status, 0, sizeof(int), s));
+  if (iters_out) *iters_out = it;
+  if (err_out) *err_out = r.err;
+  if (r.status & ST_TIMEOUT) {
+    set_error("fa_sinkhorn: a bounded device-side wait gave up (this call or an "
+              "earlier asynchronous call on the context); results are not valid");
+    return FA_ERR_TIMEOUT;
+  }
+  if (r.status & ST_NUMERIC) {
+    set_error("fa_sinkhorn: NaN/Inf or an all-zero row or column");
+    return FA_ERR_NUMERIC;
+  }
+  if (tol >= 0.0 && !(r.err <= tol)) {
+    set_error("fa_sinkhorn: err %.3e > tol %.3e after %d iterations", r.err, tol, it);
+    return FA_ERR_NOT_CONVERGED;
+  }
+  return FA_OK;
+}
+
 fa_status fa_sinkhorn(fa_ctx* c, const void* K, float* log_u, float* log_v,
                       const float* warm_log_v, int32_t max_iter, double tol,
                       int32_t check_every, int32_t* iters_out, double* err_out,
@@ -507,18 +553,31 @@ fa_status fa_sinkhorn(fa_ctx* c, const void* K, float* log_u, float* log_v,
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const bool bf16 = is_bf16(c);
   const int n1 = c->n1, n2 = c->n2;
-  SweepPlan sp = plan_sweep(n1, c->ld, bf16, c->G_sweep);
-  if (warm_log_v)
-    FA_CUDA(cudaMemcpyAsync(log_v, warm_log_v, n2 * sizeof(float), cudaMemcpyDeviceToDevice, s));
   // c->status is not cleared here: bits set by earlier asynchronous calls on
   // this context (a bounded wait in the node-cost GEMM, a non-finite row in
   // Pass B) are reported by this call, which clears them once read.
+  const bool small = c->small_C > 0 && !sweep_forced(c);
+  if (small) {
+    // every iteration of every solve has a tag of its own; start again (from
+    // cleared words) before the 32 bits run out
+    if (c->small_tag > UINT32_MAX - (uint32_t)max_iter - 1u) {
+      FA_CUDA(cudaMemsetAsync(c->small_words, 0, solve_small_words(c->small_C, c->ld), s));
+      c->small_tag = 0;
+    }
+    const uint32_t tag0 = c->small_tag;
+    c->small_tag += (uint32_t)max_iter;
+    FA_TRY(launch_solve_small(c->small_C, n1, n2, c->ld, K, bf16, warm_log_v ? warm_log_v : log_v,
+                              log_u, log_v, max_iter, tol, check_every, c->small_words, tag0,
+                              c->err, &c->result->iters, c->status, s));
+    return finish_solve(c, 0, tol, iters_out, err_out, s);
+  }
+  SweepPlan sp = plan_sweep(n1, c->ld, bf16, c->G_sweep);
+  if (warm_log_v)
+    FA_CUDA(cudaMemcpyAsync(log_v, warm_log_v, n2 * sizeof(float), cudaMemcpyDeviceToDevice, s));
   const float mu = 1.0f / (float)n1, nu = 1.0f / (float)n2;
   float* bufs[3] = {log_v, c->logv_buf[0], c->logv_buf[1]};
   int cur = 0;
-  double err = -1.0;
   int it = 0;
-  bool converged = false;
   if (c->timing && (int)c->sweep_events.size() < 2 * max_iter) {
     while ((int)c->sweep_events.size() < 2 * max_iter) {
       cudaEvent_t ev;
@@ -538,8 +597,7 @@ fa_status fa_sinkhorn(fa_ctx* c, const void* K, float* log_u, float* log_v,
     if (check) {
       FA_CUDA(cudaMemcpyAsync(&c->host_err, c->err, sizeof(double), cudaMemcpyDeviceToHost, s));
       FA_CUDA(cudaStreamSynchronize(s));
-      err = c->host_err;
-      if (err <= tol) { converged = true; break; }
+      if (c->host_err <= tol) break;
     }
     if (it == max_iter) break;   // state = (a_t in bufs[cur], b_t in log_u)
     cur = next;
@@ -547,13 +605,7 @@ fa_status fa_sinkhorn(fa_ctx* c, const void* K, float* log_u, float* log_v,
   if (it > max_iter) it = max_iter;
   if (cur != 0)
     FA_CUDA(cudaMemcpyAsync(log_v, bufs[cur], n2 * sizeof(float), cudaMemcpyDeviceToDevice, s));
-  int host_status = 0;
-  FA_CUDA(cudaMemcpyAsync(&c->host_err, c->err, sizeof(double), cudaMemcpyDeviceToHost, s));
-  FA_CUDA(cudaMemcpyAsync(&c->host_status, c->status, sizeof(int), cudaMemcpyDeviceToHost, s));
-  FA_CUDA(cudaStreamSynchronize(s));
-  err = c->host_err;
-  host_status = c->host_status;
-  if (host_status != 0) FA_CUDA(cudaMemsetAsync(c->status, 0, sizeof(int), s));
+  fa_status st = finish_solve(c, it, tol, iters_out, err_out, s);
   if (c->timing) {
     double tot = 0.0;
     for (int t = 0; t < it; ++t) {
@@ -564,22 +616,7 @@ fa_status fa_sinkhorn(fa_ctx* c, const void* K, float* log_u, float* log_v,
     c->last_sweep_ms = tot / std::max(1, it);
     c->last_sweep_n = it;
   }
-  if (iters_out) *iters_out = it;
-  if (err_out) *err_out = err;
-  if (host_status & ST_TIMEOUT) {
-    set_error("fa_sinkhorn: a bounded device-side wait gave up (this call or an "
-              "earlier asynchronous call on the context); results are not valid");
-    return FA_ERR_TIMEOUT;
-  }
-  if (host_status & ST_NUMERIC) {
-    set_error("fa_sinkhorn: NaN/Inf or an all-zero row or column");
-    return FA_ERR_NUMERIC;
-  }
-  if (tol >= 0.0 && !converged) {
-    set_error("fa_sinkhorn: err %.3e > tol %.3e after %d iterations", err, tol, it);
-    return FA_ERR_NOT_CONVERGED;
-  }
-  return FA_OK;
+  return st;
 }
 
 // ------------------------------------------------------------ read-out

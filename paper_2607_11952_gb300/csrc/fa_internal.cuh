@@ -148,6 +148,14 @@ fa_status launch_sweep(const SweepPlan& sp, int n1, int n2, int64_t ld,
                        cudaStream_t s);
 int sweep_max_active_clusters(const SweepPlan& sp, bool bf16);
 int col_finalize_max_blocks(int n2);
+// one-launch solve of small problems (k_solve_small.cu)
+int solve_small_clusters(int n1, int64_t ld, bool bf16);
+// bytes of its exchange words (0 at first); tags grow from one solve to the next
+inline size_t solve_small_words(int C, int64_t ld) { return (size_t)2 * C * ld * 8; }
+fa_status launch_solve_small(int C, int n1, int n2, int64_t ld, const void* K, bool bf16,
+                             const float* log_v_in, float* log_u, float* log_v_out, int max_iter,
+                             double tol, int check_every, void* words, uint32_t tag0,
+                             double* err, int* iters, int* status, cudaStream_t s);
 fa_status launch_col_finalize(int n2, int64_t ld, int G, const float* colpart,
                               const float* log_v_cur, float nu,
                               float* log_v_next, double* err_part,
@@ -180,6 +188,12 @@ fa_status launch_rank(int n2, int64_t ld, const void* K, bool bf16,
 }  // namespace fa
 
 // ------------------------------------------------------------ handles
+struct SolveResult {
+  double err;
+  int32_t status;
+  int32_t iters;     // of a one-launch solve
+};
+
 struct fa_graph {
   fa::DevGraph d;
 };
@@ -211,15 +225,19 @@ struct fa_ctx {
   int32_t n_anchor = 0;
   double* err_part = nullptr;     // per finalize block
   unsigned* ticket = nullptr;
-  double* err = nullptr;          // device scalar
+  SolveResult* result = nullptr;  // device: what a solve reports (err, status, iters)
+  double* err = nullptr;          // = &result->err
   double* diff = nullptr;         // plan-change block sums + result
-  int* status = nullptr;          // device status word
+  int* status = nullptr;          // = &result->status, the device status word
+  char* small_words = nullptr;    // exchange words of the one-launch solve
+  uint32_t small_tag = 0;         // tags used so far
+  int small_C = 0;                // its clusters; 0: K does not fit
   int64_t ws_bytes = 0;
   // timing
   int G_sweep = 1;                // co-resident clusters of the sweep
   int anc_cap = 1;                // capacity of anc_col
   double host_err = 0.0;
-  int host_status = 0;
+  SolveResult host_result{};
   // timing
   int timing = 0;
   double last_sweep_ms = 0.0;
