@@ -24,9 +24,10 @@ constexpr int kOffB1 = kFin * kHid;
 constexpr int kOffW2 = kOffB1 + kHid;
 constexpr int kOffC = kOffW2 + kHid;
 
-// workspace (floats): AF n*kFin | A1 n*64 | z2 n | g n | gz2 n | partials nb*kNP | scal 8
+// workspace (floats): AF n*kFin | A1 n*64 | z2 n | g n | partials nb*kNP | scal 8
+// (and n spare)
 struct GnnWs {
-  float *AF, *A1, *z2, *g, *gz2, *part, *scal;
+  float *AF, *A1, *z2, *g, *part, *scal;
   int nb;
 };
 constexpr int kGradThreads = 256;
@@ -40,8 +41,7 @@ static GnnWs ws_layout(float* w, int n) {
   s.A1 = s.AF + (size_t)n * kFin;
   s.z2 = s.A1 + (size_t)n * kHid;
   s.g = s.z2 + n;
-  s.gz2 = s.g + n;
-  s.part = s.gz2 + n;
+  s.part = s.g + n;
   s.nb = grad_blocks(n);
   s.scal = s.part + (size_t)s.nb * kNP;
   return s;
@@ -51,32 +51,74 @@ int64_t gnn_workspace_floats(int n) {
 }
 
 // ------------------------------------------------------------ reductions
+// The sums over nodes run in one block, and one SM adds only a few float64
+// numbers per clock: the float64 forms of these kernels took 11 to 37 us at
+// 4,000 to 5,000 nodes.  A sum is therefore kept as an unevaluated pair of
+// floats (Knuth's two-sum; the pair carries about 48 bits), products as the
+// float product and its exact remainder, and only the 32 warps' sums are
+// added in float64.
+struct PairSum {
+  float hi = 0.f, lo = 0.f;
+  __device__ __forceinline__ void add(float x) {
+    const float s = __fadd_rn(hi, x), b = __fsub_rn(s, hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(x, b)));
+    hi = s;
+  }
+  // + (a + da) (b + db), da and db the small parts of a pair
+  __device__ __forceinline__ void add_product(float a, float da, float b, float db) {
+    const float p = __fmul_rn(a, b);
+    add(p);
+    lo += __fmaf_rn(a, b, -p) + (a * db + da * b);
+  }
+};
+// (a - m) as a pair, m = mh + ml
+__device__ __forceinline__ void centre(float a, float mh, float ml, float& d, float& dd) {
+  d = __fsub_rn(a, mh);
+  const float t = __fsub_rn(d, a);
+  dd = __fsub_rn(__fsub_rn(__fsub_rn(a, __fsub_rn(d, t)), __fadd_rn(mh, t)), ml);
+}
+
+// Sum over a block of 1,024 threads, in every thread (fixed order: a tree
+// inside the warps, then a tree over the warps' sums)
+__device__ __forceinline__ double block_sum(PairSum x, double* warp_sums) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float h = __shfl_xor_sync(0xffffffffu, x.hi, o), l = __shfl_xor_sync(0xffffffffu, x.lo, o);
+    // the same sum in both lanes: the remainder's terms do not depend on the order
+    const float s = __fadd_rn(x.hi, h), b = __fsub_rn(s, x.hi);
+    const float e = __fadd_rn(__fsub_rn(x.hi, __fsub_rn(s, b)), __fsub_rn(h, b));
+    x.lo = __fadd_rn(__fadd_rn(x.lo, l), e);
+    x.hi = s;
+  }
+  __syncthreads();                       // warp_sums of the sum before are read
+  if ((threadIdx.x & 31) == 0) warp_sums[threadIdx.x >> 5] = (double)x.hi + (double)x.lo;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    double t = warp_sums[threadIdx.x];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (threadIdx.x == 0) warp_sums[0] = t;
+  }
+  __syncthreads();
+  return warp_sums[0];
+}
+
 // one block: out[0] = mean of x; when y (z) != null, out[1] (out[2]) = mean
 // of y (z)
 __global__ void __launch_bounds__(1024) k_means(int n, const float* __restrict__ x,
                                                 const float* __restrict__ y,
                                                 const float* __restrict__ z, float* out) {
-  __shared__ double sx[32], sy[32], sz[32];
-  double ax = 0.0, ay = 0.0, az = 0.0;
+  __shared__ double ws[32];
+  PairSum ax, ay, az;
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    ax += x[i];
-    if (y) ay += y[i];
-    if (z) az += z[i];
+    ax.add(x[i]);
+    if (y) ay.add(y[i]);
+    if (z) az.add(z[i]);
   }
-  for (int o = 16; o > 0; o >>= 1) {
-    ax += __shfl_xor_sync(0xffffffffu, ax, o);
-    ay += __shfl_xor_sync(0xffffffffu, ay, o);
-    az += __shfl_xor_sync(0xffffffffu, az, o);
-  }
-  if ((threadIdx.x & 31) == 0) {
-    sx[threadIdx.x >> 5] = ax;
-    sy[threadIdx.x >> 5] = ay;
-    sz[threadIdx.x >> 5] = az;
-  }
-  __syncthreads();
+  const double tx = block_sum(ax, ws);
+  const double ty = y ? block_sum(ay, ws) : 0.0;
+  const double tz = z ? block_sum(az, ws) : 0.0;
   if (threadIdx.x == 0) {
-    double tx = 0.0, ty = 0.0, tz = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) { tx += sx[w]; ty += sy[w]; tz += sz[w]; }
     out[0] = (float)(tx / n);
     if (y) out[1] = (float)(ty / n);
     if (z) out[2] = (float)(tz / n);
@@ -103,37 +145,39 @@ __global__ void k_gnn_features(int n, const int32_t* __restrict__ rp, const floa
 }
 
 // ------------------------------------------------------------ forward
-// AF[i] = sum_k Abar[i,k] F[k]  (thread per node)
-__global__ void k_gnn_agg(int n, const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
-                          const float* __restrict__ val, const float* __restrict__ F,
-                          float* __restrict__ AF) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  float a[kFin];
-#pragma unroll
-  for (int f = 0; f < kFin; ++f) a[f] = 0.f;
-  for (int e = rp[i]; e < rp[i + 1]; ++e) {
-    const float w = val[e];
-    const float* fk = F + (size_t)ci[e] * kFin;
-#pragma unroll
-    for (int f = 0; f < kFin; ++f) a[f] += w * fk[f];
-  }
-#pragma unroll
-  for (int f = 0; f < kFin; ++f) AF[(size_t)i * kFin + f] = a[f];
-}
-
-// A1 = AF W1 + b1, z2 = relu(A1) w2  (warp per node, two hidden units per lane)
-__global__ void __launch_bounds__(256) k_gnn_hidden(int n, const float* __restrict__ AF,
+// AF[i] = sum_k Abar[i,k] F[k], A1 = AF W1 + b1, z2 = relu(A1) w2: one warp
+// per node, the lanes over its edges, then over the hidden units (two per
+// lane).  One thread per node walked a hub's 700 edges alone (26 us at 4,000
+// nodes, and the hidden layer was a second launch); 4.6 us together now.
+__global__ void __launch_bounds__(256) k_gnn_hidden(int n, const int32_t* __restrict__ rp,
+                                                    const int32_t* __restrict__ ci,
+                                                    const float* __restrict__ val,
+                                                    const float* __restrict__ F,
                                                     const __nv_bfloat16* __restrict__ W1,
                                                     const float* __restrict__ theta,
                                                     const __nv_bfloat16* __restrict__ w2,
+                                                    float* __restrict__ AF,
                                                     float* __restrict__ A1, float* __restrict__ z2) {
   const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (i >= n) return;
   float fi[kFin];
 #pragma unroll
-  for (int f = 0; f < kFin; ++f) fi[f] = AF[(size_t)i * kFin + f];
+  for (int f = 0; f < kFin; ++f) fi[f] = 0.f;
+#pragma unroll 2
+  for (int e = rp[i] + lane, e1 = rp[i + 1]; e < e1; e += 32) {
+    const float w = val[e];
+    const float* fk = F + (size_t)ci[e] * kFin;
+#pragma unroll
+    for (int f = 0; f < kFin; ++f) fi[f] += w * fk[f];
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+    for (int f = 0; f < kFin; ++f) fi[f] += __shfl_xor_sync(0xffffffffu, fi[f], o);
+#pragma unroll
+  for (int f = 0; f < kFin; ++f)
+    if (lane == f) AF[(size_t)i * kFin + f] = fi[f];
   float z = 0.f;
 #pragma unroll
   for (int q = 0; q < 2; ++q) {
@@ -148,52 +192,74 @@ __global__ void __launch_bounds__(256) k_gnn_hidden(int n, const float* __restri
   if (lane == 0) z2[i] = z;
 }
 
-// out[i] = sum_k val[e] x[k] (+ theta[kOffC] when add_c)  (thread per node)
-__global__ void k_gnn_spmv(int n, const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
-                           const float* __restrict__ val, const float* __restrict__ x,
-                           const float* __restrict__ theta, int add_c, float* __restrict__ out) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
+// sum_k val[e] x[k] over node i's edges, in every lane of the warp
+__device__ __forceinline__ float gather_sum(int e0, int e1, int lane, const int32_t* ci,
+                                            const float* val, const float* x) {
   float s = 0.f;
-  for (int e = rp[i]; e < rp[i + 1]; ++e) s += val[e] * x[ci[e]];
-  out[i] = s + (add_c ? theta[kOffC] : 0.f);
+#pragma unroll 2
+  for (int e = e0 + lane; e < e1; e += 32) s += val[e] * x[ci[e]];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  return s;
+}
+
+// out[i] = sum_k val[e] x[k] + theta[kOffC]  (warp per node)
+__global__ void __launch_bounds__(256) k_gnn_out(int n, const int32_t* __restrict__ rp,
+                                                 const int32_t* __restrict__ ci,
+                                                 const float* __restrict__ val,
+                                                 const float* __restrict__ x,
+                                                 const float* __restrict__ theta,
+                                                 float* __restrict__ out) {
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (i >= n) return;
+  const float s = gather_sum(rp[i], rp[i + 1], lane, ci, val, x);
+  if (lane == 0) out[i] = s + theta[kOffC];
 }
 
 // ------------------------------------------------------------ backward
-// one block: residual r, g = 2 r / n, loss = mean r^2, dL/dc = sum g
+// one block: residual r = (a - y) - mean(a - y), g = 2 r / n, loss = mean r^2,
+// dL/dc = sum g
 __global__ void __launch_bounds__(1024) k_gnn_resid(int n, const float* __restrict__ a,
                                                     const float* __restrict__ y,
-                                                    const float* __restrict__ means,
                                                     float* __restrict__ g, float* loss,
                                                     float* __restrict__ grad) {
-  __shared__ double sl[32], sg[32];
-  double al = 0.0, ag = 0.0;
-  const float ma = means[0], my = means[1];
+  __shared__ double ws[32];
+  PairSum sa, sy;
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    const float r = (a[i] - ma) - (y[i] - my);
+    sa.add(a[i]);
+    sy.add(y[i]);
+  }
+  const double m = (block_sum(sa, ws) - block_sum(sy, ws)) / n;
+  const float mh = (float)m, ml = (float)(m - (double)mh);
+  PairSum sl, sg;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    // a - y as a pair, then minus the mean
+    const float d = __fsub_rn(a[i], y[i]), t = __fsub_rn(d, a[i]);
+    const float dd = __fsub_rn(__fsub_rn(a[i], __fsub_rn(d, t)), __fadd_rn(y[i], t));
+    float c, dc;
+    centre(d, mh, ml, c, dc);
+    const float r = c + (dc + dd);
     const float gi = 2.f * r / (float)n;
     g[i] = gi;
-    al += (double)r * r;
-    ag += gi;
+    sl.add_product(r, 0.f, r, 0.f);
+    sg.add(gi);
   }
-  for (int o = 16; o > 0; o >>= 1) {
-    al += __shfl_xor_sync(0xffffffffu, al, o);
-    ag += __shfl_xor_sync(0xffffffffu, ag, o);
-  }
-  if ((threadIdx.x & 31) == 0) { sl[threadIdx.x >> 5] = al; sg[threadIdx.x >> 5] = ag; }
-  __syncthreads();
+  const double al = block_sum(sl, ws), ag = block_sum(sg, ws);
   if (threadIdx.x == 0) {
-    double tl = 0.0, tg = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) { tl += sl[w]; tg += sg[w]; }
-    if (loss) *loss = (float)(tl / n);
-    grad[kOffC] = (float)tg;
+    if (loss) *loss = (float)(al / n);
+    grad[kOffC] = (float)ag;
   }
 }
 
-// per-block partial gradients of W1, b1, w2 (warp per node, 4 nodes per warp)
+// a = Abar z2 + c  =>  gz2 = dL/dz2 = Abar^T g (Abar^T[i,k] = 1/deg k), and
+// the per-block partial gradients of W1, b1, w2 (warp per node, 4 nodes per
+// warp: the node's edges over the lanes, then two hidden units per lane)
 __global__ void __launch_bounds__(kGradThreads) k_gnn_grad_part(
-    int n, const float* __restrict__ AF, const float* __restrict__ A1,
-    const __nv_bfloat16* __restrict__ w2, const float* __restrict__ gz2, float* __restrict__ part) {
+    int n, const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
+    const float* __restrict__ val, const float* __restrict__ g, const float* __restrict__ AF,
+    const float* __restrict__ A1, const __nv_bfloat16* __restrict__ w2,
+    float* __restrict__ part) {
   __shared__ float red[kGradThreads / 32][kNP - 1];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float dW[kFin][2], db[2] = {0.f, 0.f}, dw[2] = {0.f, 0.f};
@@ -204,7 +270,7 @@ __global__ void __launch_bounds__(kGradThreads) k_gnn_grad_part(
   for (int k = 0; k < 4; ++k) {
     const int i = base + k;
     if (i >= n) break;
-    const float gi = gz2[i];
+    const float gi = gather_sum(rp[i], rp[i + 1], lane, ci, val, g);
     float af[kFin];
 #pragma unroll
     for (int f = 0; f < kFin; ++f) af[f] = AF[(size_t)i * kFin + f];
@@ -235,12 +301,27 @@ __global__ void __launch_bounds__(kGradThreads) k_gnn_grad_part(
   }
 }
 
-__global__ void k_gnn_grad_reduce(int nb, const float* __restrict__ part, float* __restrict__ grad) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= kNP - 1) return;
+// grad[p] = sum over the blocks' partials: 32 parameters per block, the
+// partials over 32 groups of lanes (b = group, + 32, ...), the groups added
+// in order
+__global__ void __launch_bounds__(1024) k_gnn_grad_reduce(int nb, const float* __restrict__ part,
+                                                          float* __restrict__ grad) {
+  __shared__ float red[32][33];
+  const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
+  const int p = blockIdx.x * 32 + lane;
   float s = 0.f;
-  for (int b = 0; b < nb; ++b) s += part[(size_t)b * kNP + p];
-  grad[p] = s;
+  if (p < kNP - 1) {
+#pragma unroll 4
+    for (int b = grp; b < nb; b += 32) s += part[(size_t)b * kNP + p];
+  }
+  red[grp][lane] = s;
+  __syncthreads();
+  if (grp == 0 && p < kNP - 1) {
+    float t = 0.f;
+#pragma unroll
+    for (int k = 0; k < 32; ++k) t += red[k][lane];
+    grad[p] = t;
+  }
 }
 
 // ------------------------------------------------------------ optimiser
@@ -290,49 +371,26 @@ __global__ void __launch_bounds__(1024) k_gnn_fit_scale(int n, const float* __re
                                                         const float* __restrict__ y,
                                                         float max_abs, int shrink,
                                                         float* __restrict__ out) {
-  __shared__ double s1[32], s2[32], s3[32];
-  __shared__ double mp, my;
-  double ap = 0.0, ay = 0.0;
+  __shared__ double ws[32];
+  PairSum sp, sy;
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    ap += clamp_pred(pred[i], max_abs);
-    ay += y[i];
+    sp.add(clamp_pred(pred[i], max_abs));
+    sy.add(y[i]);
   }
-  for (int o = 16; o > 0; o >>= 1) {
-    ap += __shfl_xor_sync(0xffffffffu, ap, o);
-    ay += __shfl_xor_sync(0xffffffffu, ay, o);
-  }
-  if ((threadIdx.x & 31) == 0) { s1[threadIdx.x >> 5] = ap; s2[threadIdx.x >> 5] = ay; }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double tp = 0.0, ty = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) { tp += s1[w]; ty += s2[w]; }
-    mp = tp / n;
-    my = ty / n;
-  }
-  __syncthreads();
-  double cxy = 0.0, cxx = 0.0, cyy = 0.0;
+  const double mp = block_sum(sp, ws) / n, my = block_sum(sy, ws) / n;
+  const float ph = (float)mp, pl = (float)(mp - (double)ph);
+  const float yh = (float)my, yl = (float)(my - (double)yh);
+  PairSum sxy, sxx, syy;
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    const double dp = clamp_pred(pred[i], max_abs) - mp;
-    const double dy = (double)y[i] - my;
-    cxy += dp * dy;
-    cxx += dp * dp;
-    cyy += dy * dy;
+    float p, dp, v, dv;
+    centre(clamp_pred(pred[i], max_abs), ph, pl, p, dp);
+    centre(y[i], yh, yl, v, dv);
+    sxy.add_product(p, dp, v, dv);
+    sxx.add_product(p, dp, p, dp);
+    syy.add_product(v, dv, v, dv);
   }
-  for (int o = 16; o > 0; o >>= 1) {
-    cxy += __shfl_xor_sync(0xffffffffu, cxy, o);
-    cxx += __shfl_xor_sync(0xffffffffu, cxx, o);
-    cyy += __shfl_xor_sync(0xffffffffu, cyy, o);
-  }
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) {
-    s1[threadIdx.x >> 5] = cxy;
-    s2[threadIdx.x >> 5] = cxx;
-    s3[threadIdx.x >> 5] = cyy;
-  }
-  __syncthreads();
+  const double txy = block_sum(sxy, ws), txx = block_sum(sxx, ws), tyy = block_sum(syy, ws);
   if (threadIdx.x == 0) {
-    double txy = 0.0, txx = 0.0, tyy = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) { txy += s1[w]; txx += s2[w]; tyy += s3[w]; }
     double a = txx > 0.0 ? txy / txx : 0.0;
     a = a < 0.0 ? 0.0 : (a > 1.0 ? 1.0 : a);
     const double r2 = (txx > 0.0 && tyy > 0.0) ? (txy * txy) / (txx * tyy) : 0.0;
@@ -442,13 +500,12 @@ fa_status fa_gnn_forward(fa_gnn* g, const fa_graph* graph, const float* F, float
   const DevGraph& d = graph->d;
   const int n = d.n;
   GnnWs w = ws_layout(ws, n);
-  k_gnn_agg<<<(n + 255) / 256, 256, 0, s>>>(n, d.row_ptr, d.col, d.val_row, F, w.AF);
-  FA_LAUNCHED("k_gnn_agg");
-  k_gnn_hidden<<<(unsigned)(((int64_t)n * 32 + 255) / 256), 256, 0, s>>>(n, w.AF, g->W1, g->theta,
-                                                                          g->w2, w.A1, w.z2);
+  const unsigned blocks = (unsigned)(((int64_t)n * 32 + 255) / 256);   // a warp per node
+  k_gnn_hidden<<<blocks, 256, 0, s>>>(n, d.row_ptr, d.col, d.val_row, F, g->W1, g->theta, g->w2,
+                                      w.AF, w.A1, w.z2);
   FA_LAUNCHED("k_gnn_hidden");
-  k_gnn_spmv<<<(n + 255) / 256, 256, 0, s>>>(n, d.row_ptr, d.col, d.val_row, w.z2, g->theta, 1, a_out);
-  FA_LAUNCHED("k_gnn_spmv");
+  k_gnn_out<<<blocks, 256, 0, s>>>(n, d.row_ptr, d.col, d.val_row, w.z2, g->theta, a_out);
+  FA_LAUNCHED("k_gnn_out");
   return FA_OK;
 }
 
@@ -462,16 +519,12 @@ fa_status fa_gnn_backward(fa_gnn* g, const fa_graph* graph, const float* ws_in, 
   const DevGraph& d = graph->d;
   const int n = d.n;
   GnnWs w = ws_layout(const_cast<float*>(ws_in), n);
-  k_means<<<1, 1024, 0, s>>>(n, a_pred, target, nullptr, w.scal);
-  FA_LAUNCHED("k_means");
-  k_gnn_resid<<<1, 1024, 0, s>>>(n, a_pred, target, w.scal, w.g, loss, grad);
+  k_gnn_resid<<<1, 1024, 0, s>>>(n, a_pred, target, w.g, loss, grad);
   FA_LAUNCHED("k_gnn_resid");
-  // a = Abar z2 + c  =>  dL/dz2 = Abar^T g (Abar^T[i,k] = 1/deg k)
-  k_gnn_spmv<<<(n + 255) / 256, 256, 0, s>>>(n, d.row_ptr, d.col, d.val_col, w.g, g->theta, 0, w.gz2);
-  FA_LAUNCHED("k_gnn_spmv");
-  k_gnn_grad_part<<<w.nb, kGradThreads, 0, s>>>(n, w.AF, w.A1, g->w2, w.gz2, w.part);
+  k_gnn_grad_part<<<w.nb, kGradThreads, 0, s>>>(n, d.row_ptr, d.col, d.val_col, w.g, w.AF, w.A1,
+                                                g->w2, w.part);
   FA_LAUNCHED("k_gnn_grad_part");
-  k_gnn_grad_reduce<<<(kNP + 255) / 256, 256, 0, s>>>(w.nb, w.part, grad);
+  k_gnn_grad_reduce<<<(kNP - 1 + 31) / 32, 1024, 0, s>>>(w.nb, w.part, grad);
   FA_LAUNCHED("k_gnn_grad_reduce");
   return FA_OK;
 }
