@@ -680,27 +680,35 @@ SweepPlan plan_sweep(int n1, int64_t ld, bool bf16, int max_G) {
   // ld; W is the widest slab.  A step costs a fixed part (barriers, the
   // exchange) plus a part per round of NT vectors, so a shape should have
   // few rounds, a nearly full last round and, where the ring allows, two
-  // rows per step.  BF16 default rule (measured on GB300, 50,000 rows and
-  // 30k-110k columns: it picks the fastest of the rules below at every
-  // width):
-  //   1. the smallest power-of-two cluster up to 8 whose slab takes at most
+  // rows per step.  BF16 default rule, each line
+  // where the shapes above it do not fit (measured on GB300, fraction of the
+  // copy peak against the rule that began at line 3; 30k-110k columns: lines
+  // 3 to 5 pick the fastest of themselves at every width):
+  //   1. the smallest cluster up to 8 with two rows per step and four or five
+  //      nearly full rounds (88%, 86%): 18k columns 0.65 -> 0.76 (clusters of
+  //      2), 24k 0.64 -> 0.77 (3), 36k 0.70 -> 0.79 (4), 40k 0.71 -> 0.78
+  //      (5), 44k 0.63 -> 0.75 (5); at 50k six CTAs (82% full) tie with line
+  //      4's five, seven (87%) lose;
+  //   2. the smallest cluster of 2 to 4 with two rows and three full rounds
+  //      (95%): 12k 0.58 -> 0.65;
+  //   3. the smallest power-of-two cluster up to 8 whose slab takes at most
   //      5 vectors per thread with the last round at least 80% full;
-  //   2. else the smallest cluster up to 10 with at most 5 vectors;
-  //   3. else the smallest cluster of any size that fits the register
-  //      shapes.
+  //   4. the smallest cluster up to 10 with at most 5 vectors;
+  //   5. the smallest cluster of any size that fits the register shapes.
   // FP32, already at the copy peak, keeps powers of two.  FA_SWEEP_ANYQ=0
   // forces powers of two, =1 the smallest cluster of any size.
   const int64_t units = ld / V;
   const int qrule = env_int("FA_SWEEP_ANYQ", bf16 ? 2 : 0);
-  auto fit = [&](int Q, int min_ns, int s_cap, double min_fill) -> bool {
+  auto fit = [&](int Q, int min_ns, int s_cap, double min_fill, int s_min = 1,
+                 int r_min = 1) -> bool {
     if (Qforce && Q != Qforce) return false;
     if (units < Q) return false;
     const int64_t W = V * ((units + Q - 1) / Q);
     const int S = (int)((W + (int64_t)NT * V - 1) / ((int64_t)NT * V));
-    if (S > s_cap) return false;
+    if (S > s_cap || S < s_min) return false;
     if ((double)(W / V) < min_fill * (double)S * NT) return false;
     const size_t budget = kSmemBudget / sweep_ctas_per_sm(NT, S * V);
-    for (int R = bf16 ? 4 : 2; R >= 1; R /= 2) {
+    for (int R = bf16 ? 4 : 2; R >= r_min; R /= 2) {
       if (Rforce && R != Rforce) continue;
       const size_t fixed = (size_t)(kMaxNS + kNX) * 8 + (size_t)(2 * R * (NT / 32) + kNX * kMaxQ * R) * 4;
       int NS = (int)((budget - fixed) / ((size_t)R * W * b));
@@ -722,6 +730,11 @@ SweepPlan plan_sweep(int n1, int64_t ld, bool bf16, int max_G) {
     const int min_ns = pass == 0 ? 3 : 2;
     if (qrule == 2) {
       const int s5 = smax < 5 ? smax : 5;
+      if (NT == 256 && smax >= 5) {
+        for (int Q = 1; Q <= 8 && sp.Q == 0; ++Q)
+          if (!fit(Q, min_ns, 5, 0.86, 5, 2)) fit(Q, min_ns, 4, 0.88, 4, 2);
+        for (int Q = 2; Q <= 4 && sp.Q == 0; ++Q) fit(Q, min_ns, 3, 0.95, 3, 2);
+      }
       for (int Q = 1; Q <= 8 && sp.Q == 0; Q *= 2) fit(Q, min_ns, s5, 0.8);
       for (int Q = 1; Q <= 10 && sp.Q == 0; ++Q) fit(Q, min_ns, s5, 0.0);
       for (int Q = 1; Q <= kMaxQ && sp.Q == 0; ++Q) fit(Q, min_ns, smax, 0.0);
