@@ -145,7 +145,7 @@ SweepPlan plan_sweep(int n1, int64_t ld, bool bf16, int max_G);
 fa_status launch_sweep(const SweepPlan& sp, int n1, int n2, int64_t ld,
                        const void* K, bool bf16, const float* log_v,
                        float* log_u, float mu, float* colpart, int* status,
-                       cudaStream_t s);
+                       cudaStream_t s, bool reversed = false, bool overlap = false);
 int sweep_max_active_clusters(const SweepPlan& sp, bool bf16);
 int col_finalize_max_blocks(int n2);
 // one-launch solve of small problems (k_solve_small.cu)
@@ -160,7 +160,7 @@ fa_status launch_col_finalize(int n2, int64_t ld, int G, const float* colpart,
                               const float* log_v_cur, float nu,
                               float* log_v_next, double* err_part,
                               unsigned* ticket, double* err_out, int* status,
-                              cudaStream_t s);
+                              cudaStream_t s, bool overlap = false);
 
 // Column-sharded sweep (k_shard.cu)
 constexpr int kShardBlock = FA_SHARD_BLOCK;

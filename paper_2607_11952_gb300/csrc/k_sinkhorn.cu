@@ -37,6 +37,30 @@ namespace cg = cooperative_groups;
 
 namespace fa {
 
+// Programmatic dependent launch: wait for the kernel this launch may overlap
+// with (no effect in an ordinary launch), and let the next one start.
+__device__ __forceinline__ void grid_dependency_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void grid_dependency_trigger() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+// Loads of what the kernel before wrote: volatile, so that the compiler keeps
+// them behind the wait (a plain load through a const restrict pointer, or the
+// cache-hint intrinsics, may be moved before it).
+__device__ __forceinline__ float load_dependent(const float* p) {
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float4 load_dependent4(const float* p) {
+  float4 v;
+  asm volatile("ld.global.cs.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "l"(p));
+  return v;
+}
+
 // ------------------------------------------------------------ plan init
 // T0 = mu nu^T (reading: independent coupling): K = 1, log u = log mu,
 // log v = log nu.
@@ -192,8 +216,8 @@ __device__ __forceinline__ void sum_slots(const float* xs, float (&rs)[R]) {
 template <typename TK, int S, int R, int NT>
 __global__ void __launch_bounds__(NT, sweep_ctas_per_sm(NT, S * KT<TK>::V)) k_sweep(
     const TK* __restrict__ K, int64_t ld, int n1, int n2, int W, int NS,
-    const float* __restrict__ log_v, float* __restrict__ log_u, float mu,
-    float log_mu, float* __restrict__ colpart, int* __restrict__ status) {
+    const float* log_v, float* __restrict__ log_u, float mu,
+    float log_mu, float* __restrict__ colpart, int* __restrict__ status, int64_t row_step, int u_step) {
   constexpr int V = KT<TK>::V;
   constexpr int NW = NT / 32;
   extern __shared__ __align__(128) unsigned char smem[];
@@ -236,32 +260,6 @@ __global__ void __launch_bounds__(NT, sweep_ctas_per_sm(NT, S * KT<TK>::V)) k_sw
     cluster_wait();
   }
 
-  // v and the column accumulators as packed pairs (columns 2k, 2k+1)
-  constexpr int V2 = V / 2;
-  f2_t vv[S][V2], acc[S][V2];
-#pragma unroll
-  for (int s = 0; s < S; ++s) {
-    const int e0 = (s * NT + tid) * V;
-#pragma unroll
-    for (int k = 0; k < V2; ++k) {
-      const int64_t col = off + e0 + 2 * k;
-      const float a = (e0 < Wq && col < n2) ? expf(log_v[col]) : 0.f;
-      const float b = (e0 < Wq && col + 1 < n2) ? expf(log_v[col + 1]) : 0.f;
-      vv[s][k] = pk2(a, b);
-      acc[s][k] = pk2(0.f, 0.f);
-    }
-  }
-
-  // 32-bit shared addresses of this thread's vectors in a ring row.  A
-  // vector past the slab edge (e0 >= W) is read at the slab's last vector
-  // instead: its v is 0, so it adds nothing to the row sums, and its column
-  // accumulators are never stored -- so no per-vector branch is needed.
-  uint32_t voff[S];
-#pragma unroll
-  for (int s = 0; s < S; ++s) {
-    const int e0 = (s * NT + tid) * V;
-    voff[s] = (uint32_t)((e0 < Wq ? e0 : Wq - V) * (int)sizeof(TK));
-  }
   const uint32_t ring_s = smem_u32(ring);
   const uint32_t rowb = (uint32_t)W * sizeof(TK);
   // vectors s < S-1 are inside the slab for every thread; the last one only
@@ -277,11 +275,43 @@ __global__ void __launch_bounds__(NT, sweep_ctas_per_sm(NT, S * KT<TK>::V)) k_sw
     mbar_expect_tx(mb, (uint32_t)nrows * row_bytes);
     for (int r = 0; r < nrows; ++r)
       bulk_g2s(smem_u32(ring + ((size_t)stage * R + r) * W),
-               Kslab + (int64_t)(row0 + r) * ld, row_bytes, mb);
+               Kslab + (int64_t)(row0 + r) * row_step, row_bytes, mb);
   };
   if (tid == 0) {
     for (int t = 0; t < min(NS, T); ++t) issue(t, t);
     issued = min(NS, T);
+  }
+  // K was complete before the launch this one may overlap with (the previous
+  // iteration's finalisation); v comes from that launch
+  grid_dependency_wait();
+  // v and the column accumulators as packed pairs (columns 2k, 2k+1)
+  constexpr int V2 = V / 2;
+  f2_t vv[S][V2], acc[S][V2];
+#pragma unroll
+  for (int s = 0; s < S; ++s) {
+    const int e0 = (s * NT + tid) * V;
+#pragma unroll
+    for (int k = 0; k < V2; ++k) {
+      const int64_t col = off + e0 + 2 * k;
+      // unconditional loads (of a valid column), so that all are in flight together
+      const float la = load_dependent(log_v + min(col, (int64_t)n2 - 1));
+      const float lb = load_dependent(log_v + min(col + 1, (int64_t)n2 - 1));
+      const float a = (e0 < Wq && col < n2) ? expf(la) : 0.f;
+      const float b = (e0 < Wq && col + 1 < n2) ? expf(lb) : 0.f;
+      vv[s][k] = pk2(a, b);
+      acc[s][k] = pk2(0.f, 0.f);
+    }
+  }
+
+  // 32-bit shared addresses of this thread's vectors in a ring row.  A
+  // vector past the slab edge (e0 >= W) is read at the slab's last vector
+  // instead: its v is 0, so it adds nothing to the row sums, and its column
+  // accumulators are never stored -- so no per-vector branch is needed.
+  uint32_t voff[S];
+#pragma unroll
+  for (int s = 0; s < S; ++s) {
+    const int e0 = (s * NT + tid) * V;
+    voff[s] = (uint32_t)((e0 < Wq ? e0 : Wq - V) * (int)sizeof(TK));
   }
 
   bool dead = false;
@@ -412,7 +442,7 @@ __global__ void __launch_bounds__(NT, sweep_ctas_per_sm(NT, S * KT<TK>::V)) k_sw
           } else if (tid == 0) {
             atomicOr(status, ST_NUMERIC);
           }
-          if (q == 0 && tid == r) log_u[row] = log_mu - logf(rs);
+          if (q == 0 && tid == r) log_u[(int64_t)row * u_step] = log_mu - logf(rs);
         }
         u[r] = ur;
       }
@@ -453,6 +483,251 @@ __global__ void __launch_bounds__(NT, sweep_ctas_per_sm(NT, S * KT<TK>::V)) k_sw
     for (int t = max(0, issued - NS); t < issued; ++t)
       mbar_wait_bounded(smem_u32(&full[t % NS]), (uint32_t)((t / NS) & 1));
   }
+  grid_dependency_trigger();
+  if (Q > 1) {   // no CTA leaves while a peer may still address its memory
+    cluster_arrive();
+    cluster_wait();
+  }
+#pragma unroll
+  for (int s = 0; s < S; ++s) {
+    const int e0 = (s * NT + tid) * V;
+    if (e0 < Wq) {
+      float* dst = colpart + (int64_t)g * ld + off + e0;
+#pragma unroll
+      for (int k = 0; k < V2; k += 2) {
+        const float2 a = upk2(acc[s][k]), b = upk2(acc[s][k + 1]);
+        *reinterpret_cast<float4*>(dst + 2 * k) = make_float4(a.x, a.y, b.x, b.y);
+      }
+    }
+  }
+}
+
+// The same sweep with K's raw vectors carried in registers from the row pass
+// of a step to its column pass one step later: one shared load per vector
+// instead of two, a ring stage is free as soon as the row pass has read it,
+// and a step has one block barrier (its row partials) instead of two.  The
+// cluster's exchange of step t - 1 is waited for before step t's vectors are
+// read; the two CTAs of an SM cover each other's waits.  It pays where a row
+// step is long enough to cover them and the vectors fit the registers: see
+// sweep_ptr for where it is taken and what it measured.
+template <typename TK, int S, int R, int NT>
+__global__ void __launch_bounds__(NT, 2) k_sweep_reg(
+    const TK* __restrict__ K, int64_t ld, int n1, int n2, int W, int NS,
+    const float* log_v, float* __restrict__ log_u, float mu,
+    float log_mu, float* __restrict__ colpart, int* __restrict__ status, int64_t row_step, int u_step) {
+  constexpr int V = KT<TK>::V, V2 = V / 2;
+  constexpr int NW = NT / 32;
+  constexpr int kLead = NT - 32;           // the thread that feeds the ring and the slots
+  extern __shared__ __align__(128) unsigned char smem[];
+  TK* ring = reinterpret_cast<TK*>(smem);
+  const size_t ring_bytes = (size_t)NS * R * W * sizeof(TK);
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + ring_bytes);
+  uint64_t* xbar = full + kMaxNS;
+  float* red = reinterpret_cast<float*>(xbar + kNX);
+  float* xch = red + 2 * R * NW;
+  __shared__ int s_timeout;
+
+  const int Q = (int)cluster_size();
+  const int q = (int)cluster_rank();
+  const int g = blockIdx.x / Q;            // cluster = row-step group
+  const int G = gridDim.x / Q;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int nsteps = (n1 + R - 1) / R;
+  const int T = g < nsteps ? (nsteps - 1 - g) / G + 1 : 0;   // cluster-uniform
+  const int units = (int)(ld / V), ubase = units / Q, urem = units - ubase * Q;
+  const int Wq = V * (ubase + (q < urem ? 1 : 0));
+  const int64_t off = (int64_t)V * (q * ubase + min(q, urem));
+  const TK* Kslab = K + off;
+  const uint32_t row_bytes = (uint32_t)Wq * sizeof(TK);
+  const uint32_t xch_bytes = (uint32_t)(Q * R * 4);
+
+  if (tid == 0) {
+    for (int s = 0; s < NS; ++s) mbar_init(smem_u32(&full[s]), 1);
+    for (int s = 0; s < kNX; ++s) mbar_init(smem_u32(&xbar[s]), 1);
+    fence_mbar_init();
+    s_timeout = 0;
+    if (Q > 1)
+      for (int t = 0; t < min(kNX, T); ++t) mbar_expect_tx(smem_u32(&xbar[t]), xch_bytes);
+  }
+  __syncthreads();
+  if (Q > 1) {   // every CTA's barriers exist before any remote store
+    cluster_arrive();
+    cluster_wait();
+  }
+  const uint32_t ring_s = smem_u32(ring);
+  const uint32_t rowb = (uint32_t)W * sizeof(TK);
+  const bool last_ok = ((S - 1) * NT + warp * 32) * V < Wq;
+
+  int issued = 0;   // meaningful in thread kLead only
+  auto issue = [&](int t, int stage) {
+    const int row0 = (g + t * G) * R;
+    const int nrows = min(R, n1 - row0);
+    const uint32_t mb = smem_u32(&full[stage]);
+    mbar_expect_tx(mb, (uint32_t)nrows * row_bytes);
+    for (int r = 0; r < nrows; ++r)
+      bulk_g2s(smem_u32(ring + ((size_t)stage * R + r) * W),
+               Kslab + (int64_t)(row0 + r) * row_step, row_bytes, mb);
+  };
+  if (tid == kLead) {
+    for (int t = 0; t < min(NS, T); ++t) issue(t, t);
+    issued = min(NS, T);
+  }
+  // K was complete before the launch this one may overlap with (the previous
+  // iteration's finalisation); v comes from that launch
+  grid_dependency_wait();
+  f2_t vv[S][V2], acc[S][V2];
+  uint4 raw[R][S];
+  uint32_t voff[S];
+#pragma unroll
+  for (int s = 0; s < S; ++s) {
+    const int e0 = (s * NT + tid) * V;
+#pragma unroll
+    for (int k = 0; k < V2; ++k) {
+      const int64_t col = off + e0 + 2 * k;
+      // unconditional loads (of a valid column), so that all are in flight together
+      const float la = load_dependent(log_v + min(col, (int64_t)n2 - 1));
+      const float lb = load_dependent(log_v + min(col + 1, (int64_t)n2 - 1));
+      const float a = (e0 < Wq && col < n2) ? expf(la) : 0.f;
+      const float b = (e0 < Wq && col + 1 < n2) ? expf(lb) : 0.f;
+      vv[s][k] = pk2(a, b);
+      acc[s][k] = pk2(0.f, 0.f);
+    }
+    voff[s] = (uint32_t)((e0 < Wq ? e0 : Wq - V) * (int)sizeof(TK));
+#pragma unroll
+    for (int r = 0; r < R; ++r) raw[r][s] = make_uint4(0u, 0u, 0u, 0u);
+  }
+  bool dead = false;
+  int stage = 0;
+  uint32_t ph = 0;
+  for (int t = 0; t <= T; ++t) {
+    // -------- step t-1: full row sums and u
+    float u[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) u[r] = 0.f;
+    if (t > 0) {
+      const int tp = t - 1;
+      const int row0 = (g + tp * G) * R;
+      float rsum[R];
+      if (Q > 1) {
+        if (!dead && !mbar_wait_bounded(smem_u32(&xbar[tp % kNX]), (uint32_t)((tp / kNX) & 1))) {
+          atomicOr(status, ST_TIMEOUT);
+          s_timeout = 1;
+        }
+        const float* xs = xch + (tp % kNX) * kMaxQ * R;
+        switch (Q) {
+          case 2: sum_slots<R, 2>(xs, rsum); break;
+          case 3: sum_slots<R, 3>(xs, rsum); break;
+          case 4: sum_slots<R, 4>(xs, rsum); break;
+          case 5: sum_slots<R, 5>(xs, rsum); break;
+          case 6: sum_slots<R, 6>(xs, rsum); break;
+          case 7: sum_slots<R, 7>(xs, rsum); break;
+          case 8: sum_slots<R, 8>(xs, rsum); break;
+          case 9: sum_slots<R, 9>(xs, rsum); break;
+          case 10: sum_slots<R, 10>(xs, rsum); break;
+          case 11: sum_slots<R, 11>(xs, rsum); break;
+          case 12: sum_slots<R, 12>(xs, rsum); break;
+          case 13: sum_slots<R, 13>(xs, rsum); break;
+          case 14: sum_slots<R, 14>(xs, rsum); break;
+          case 15: sum_slots<R, 15>(xs, rsum); break;
+          default: sum_slots<R, 16>(xs, rsum); break;   // Q = 16 (kMaxQ)
+        }
+      } else {
+        const float* rbp = red + (tp & 1) * R * NW;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          rsum[r] = 0.f;
+#pragma unroll
+          for (int w = 0; w < NW; ++w) rsum[r] += rbp[r * NW + w];
+        }
+      }
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const float rs = rsum[r];
+        const int row = row0 + r;
+        if (row < n1) {
+          if (rs > 0.f && isfinite(rs)) {
+            u[r] = __fdividef(mu, rs);   // identical in every CTA of the cluster
+            if (!isfinite(u[r])) { u[r] = 0.f; atomicOr(status, ST_NUMERIC); }
+          } else if (tid == 0) {
+            atomicOr(status, ST_NUMERIC);
+          }
+          if (q == 0 && tid == r) log_u[(int64_t)row * u_step] = log_mu - logf(rs);
+        }
+      }
+    }
+    if (t < T && !dead && !mbar_wait_bounded(smem_u32(&full[stage]), ph)) {
+      atomicOr(status, ST_TIMEOUT);
+      s_timeout = 1;
+    }
+    // -------- row sums of step t from the ring, columns of step t-1 from
+    // registers (t = T: its rows lie past n1, only the columns remain)
+    const int row0 = (g + t * G) * R;
+    float* rb = red + (t & 1) * R * NW;
+    const uint32_t sb = ring_s + (uint32_t)(stage * R) * rowb;
+    float p[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const f2_t u2 = pk2(u[r], u[r]);
+      f2_t pa[2] = {pk2(0.f, 0.f), pk2(0.f, 0.f)};
+      const bool in = t < T && row0 + r < n1;
+      const uint32_t rbase = sb + (uint32_t)r * rowb;
+#pragma unroll
+      for (int s = 0; s < S; ++s) {
+        if (s + 1 < S || last_ok) {
+          const uint4 nw = in ? lds128a(rbase + voff[s]) : make_uint4(0u, 0u, 0u, 0u);
+          f2_t f[V2];
+          pairs(raw[r][s], f, TK());
+#pragma unroll
+          for (int k = 0; k < V2; ++k) acc[s][k] = ffma2(u2, f[k], acc[s][k]);
+          raw[r][s] = nw;
+          pairs(nw, f, TK());
+#pragma unroll
+          for (int k = 0; k < V2; ++k) pa[k & 1] = ffma2(f[k], vv[s][k], pa[k & 1]);
+        }
+      }
+      const float2 a = upk2(pa[0]), b = upk2(pa[1]);
+      p[r] = (a.x + a.y) + (b.x + b.y);
+    }
+    if (t == T) break;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) p[r] += __shfl_xor_sync(0xffffffffu, p[r], o);
+    }
+    if (lane == 0) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) rb[r * NW + warp] = p[r];
+    }
+    __syncthreads();   // row partials of step t; stage t and slot t-1 are consumed
+    dead = s_timeout != 0;
+    if (Q > 1 && tid < R) {
+      float sum = 0.f;
+#pragma unroll
+      for (int w = 0; w < NW; ++w) sum += rb[tid * NW + w];
+      const uint32_t slot = smem_u32(xch + ((t % kNX) * kMaxQ + q) * R + tid);
+      const uint32_t bar = smem_u32(&xbar[t % kNX]);
+      for (int dst = 0; dst < Q; ++dst)
+        st_async_f32(map_cluster(slot, (uint32_t)dst), sum, map_cluster(bar, (uint32_t)dst));
+    }
+    if (tid == kLead) {
+      if (Q > 1 && t > 0 && t - 1 + kNX < T)
+        mbar_expect_tx(smem_u32(&xbar[(t - 1) % kNX]), xch_bytes);
+      if (!dead && t + NS < T) {
+        issue(t + NS, stage);
+        issued = t + NS + 1;
+      }
+    }
+    if (++stage == NS) {
+      stage = 0;
+      ph ^= 1u;
+    }
+  }
+  // after a timeout, wait (bounded) for copies still in flight into the ring
+  if (tid == kLead && dead) {
+    for (int t = max(0, issued - NS); t < issued; ++t)
+      mbar_wait_bounded(smem_u32(&full[t % NS]), (uint32_t)((t / NS) & 1));
+  }
+  grid_dependency_trigger();
   if (Q > 1) {   // no CTA leaves while a peer may still address its memory
     cluster_arrive();
     cluster_wait();
@@ -473,6 +748,12 @@ __global__ void __launch_bounds__(NT, sweep_ctas_per_sm(NT, S * KT<TK>::V)) k_sw
 
 template <typename TK, int S, int R>
 static void* sweep_ptr(int NT) {
+  // measured (GB300, BF16): only three vectors per thread and two rows per
+  // step are faster with K carried in registers (24,000 columns in clusters
+  // of 4: 0.335 -> 0.290 ms, 12,000 in 2: 74 -> 66 us, 5,000 in 1: 20.7 ->
+  // 18.4 us); one row per step loses 10-17%, four vectors and two rows 8%
+  if constexpr (sizeof(TK) == 2 && S == 3 && R == 2)
+    if (NT == 256) return reinterpret_cast<void*>(&k_sweep_reg<TK, S, R, 256>);
   if (NT == 1024) {   // 64 registers per thread: only small slabs per thread
     if constexpr (S <= (sizeof(TK) == 2 ? 3 : 6))
       return reinterpret_cast<void*>(&k_sweep<TK, S, R, 1024>);
@@ -790,7 +1071,7 @@ static cudaError_t prepare_sweep(void* fn, const SweepPlan& sp, bool bf16) {
 fa_status launch_sweep(const SweepPlan& sp, int n1, int n2, int64_t ld,
                        const void* K, bool bf16, const float* log_v,
                        float* log_u, float mu, float* colpart, int* status,
-                       cudaStream_t s) {
+                       cudaStream_t s, bool reversed, bool overlap) {
   if (sp.Q < 1) {
     set_error("fa_sinkhorn: no cluster shape fits a row of %lld elements", (long long)ld);
     return FA_ERR_UNSUPPORTED;
@@ -805,13 +1086,35 @@ fa_status launch_sweep(const SweepPlan& sp, int n1, int n2, int64_t ld,
     set_error("k_sweep attributes: %s", cudaGetErrorString(e));
     return FA_ERR_UNSUPPORTED;
   }
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   cudaLaunchConfig_t cfg = sweep_config(sp, bf16, (unsigned)(sp.G * sp.Q), attr, s);
+  // Overlap with the finalisation before it, where the blocks are placed one
+  // or two at a time.  A larger cluster that starts while the finalisation's
+  // blocks still hold parts of the SMs finds no room for itself in one place:
+  // the last clusters then wait for a whole sweep (24,000 columns in clusters
+  // of 3: 292 -> 511 us per iteration, 40,000 in 5: 630 -> 1149).  With it:
+  // 5,000 FP32 31.6 -> 25.4 us, 10,000 81.6 -> 75.7, 20,000 BF16 188 -> 183.
+  if (overlap && sp.kind == 0 && sp.Q <= 2) {
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.numAttrs = 2;
+  }
   const float log_mu = logf(mu);
   int W = sp.W, NS = sp.NS, L = sp.L;
+  // last row first: the kernel's row i is row n1 - 1 - i (the same code, with
+  // negative steps; an index chosen in the kernel cost it 6% at 50,000 columns)
+  int64_t row_step = ld;
+  int u_step = 1;
+  if (reversed && sp.kind == 0) {
+    K = static_cast<const char*>(K) + (int64_t)(n1 - 1) * ld * (bf16 ? 2 : 4);
+    log_u += n1 - 1;
+    row_step = -ld;
+    u_step = -1;
+  }
   void* args[] = {(void*)&K, (void*)&ld, (void*)&n1, (void*)&n2, (void*)&W,
                   (void*)&NS, (void*)&log_v, (void*)&log_u, (void*)&mu,
-                  (void*)&log_mu, (void*)&colpart, (void*)&status};
+                  (void*)&log_mu, (void*)&colpart, (void*)&status, (void*)&row_step,
+                  (void*)&u_step};
   void* args_ws[] = {(void*)&K, (void*)&ld, (void*)&n1, (void*)&n2, (void*)&W,
                      (void*)&NS, (void*)&L, (void*)&log_v, (void*)&log_u, (void*)&mu,
                      (void*)&log_mu, (void*)&colpart, (void*)&status};
@@ -876,8 +1179,8 @@ constexpr int kFinNarrow = 16384;
 
 template <int LC>
 __global__ void __launch_bounds__(kFinThreads) k_col_finalize(
-    int n2, int64_t ld, int G, const float* __restrict__ colpart,
-    const float* __restrict__ log_v_cur, float nu, float log_nu,
+    int n2, int64_t ld, int G, const float* colpart,
+    const float* log_v_cur, float nu, float log_nu,
     float* __restrict__ log_v_next, double* __restrict__ err_part,
     unsigned* __restrict__ ticket, double* __restrict__ err_out,
     int* __restrict__ status) {
@@ -887,6 +1190,8 @@ __global__ void __launch_bounds__(kFinThreads) k_col_finalize(
   __shared__ bool last;
   const int lc = threadIdx.x % LC, rg = threadIdx.x / LC;
   const int jb = blockIdx.x * C;
+  grid_dependency_wait();
+  grid_dependency_trigger();   // the next sweep may load its first rows of K
   {
     float4 cs = make_float4(0.f, 0.f, 0.f, 0.f);
     if (jb + 4 * lc < n2) {
@@ -896,14 +1201,14 @@ __global__ void __launch_bounds__(kFinThreads) k_col_finalize(
         float4 a[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k)
-          a[k] = __ldcs(reinterpret_cast<const float4*>(p + (int64_t)(g + k * RG) * ld));
+          a[k] = load_dependent4(p + (int64_t)(g + k * RG) * ld);
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
           cs.x += a[k].x; cs.y += a[k].y; cs.z += a[k].z; cs.w += a[k].w;
         }
       }
       for (; g < G; g += RG) {
-        const float4 a = __ldcs(reinterpret_cast<const float4*>(p + (int64_t)g * ld));
+        const float4 a = load_dependent4(p + (int64_t)g * ld);
         cs.x += a.x; cs.y += a.y; cs.z += a.z; cs.w += a.w;
       }
     }
@@ -917,7 +1222,7 @@ __global__ void __launch_bounds__(kFinThreads) k_col_finalize(
 #pragma unroll
     for (int r = 0; r < RG; ++r) c += part[r][threadIdx.x];
     if (log_v_cur) {
-      const double m = (double)expf(log_v_cur[j]) * (double)c;
+      const double m = (double)expf(load_dependent(log_v_cur + j)) * (double)c;
       e = fabs(m - (double)nu);
     }
     float lv;
@@ -976,19 +1281,27 @@ fa_status launch_col_finalize(int n2, int64_t ld, int G, const float* colpart,
                               const float* log_v_cur, float nu,
                               float* log_v_next, double* err_part,
                               unsigned* ticket, double* err_out, int* status,
-                              cudaStream_t s) {
+                              cudaStream_t s, bool overlap) {
   if ((reinterpret_cast<uintptr_t>(colpart) & 15u) != 0 || (ld & 3) != 0) {
     set_error("column finalisation: partial sums not 16-byte aligned");
     return FA_ERR_ARG;
   }
   const int C = col_finalize_cols(n2);
-  const int blocks = (n2 + C - 1) / C;
-  if (C == 32)
-    k_col_finalize<8><<<blocks, kFinThreads, 0, s>>>(n2, ld, G, colpart, log_v_cur, nu, logf(nu),
-                                                     log_v_next, err_part, ticket, err_out, status);
-  else
-    k_col_finalize<32><<<blocks, kFinThreads, 0, s>>>(n2, ld, G, colpart, log_v_cur, nu, logf(nu),
-                                                      log_v_next, err_part, ticket, err_out, status);
+  cudaLaunchAttribute attr[1];
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)((n2 + C - 1) / C));
+  cfg.blockDim = dim3(kFinThreads);
+  cfg.stream = s;
+  if (overlap) {
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+  }
+  const float log_nu = logf(nu);
+  FA_CUDA(cudaLaunchKernelEx(&cfg, C == 32 ? k_col_finalize<8> : k_col_finalize<32>, n2, ld, G,
+                             colpart, log_v_cur, nu, log_nu, log_v_next, err_part, ticket,
+                             err_out, status));
   FA_LAUNCHED("k_col_finalize");
   return FA_OK;
 }
