@@ -91,7 +91,9 @@ __device__ __forceinline__ double block_sum(PairSum x, double* warp_sums) {
     x.hi = s;
   }
   __syncthreads();                       // warp_sums of the sum before are read
-  if ((threadIdx.x & 31) == 0) warp_sums[threadIdx.x >> 5] = (double)x.hi + (double)x.lo;
+  // a sum that has left the finite numbers has no remainder
+  if ((threadIdx.x & 31) == 0)
+    warp_sums[threadIdx.x >> 5] = (double)x.hi + (isfinite(x.hi) ? (double)x.lo : 0.0);
   __syncthreads();
   if (threadIdx.x < 32) {
     double t = warp_sums[threadIdx.x];

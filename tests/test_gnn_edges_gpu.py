@@ -68,3 +68,20 @@ def test_fit_scale(n, shrink):
                            shrink=shrink)
         want = G.fit_scale(pred, y, 45.0, shrink)
         assert abs(out.item() - want) <= 2.0 ** -23 * max(1.0, want)
+
+
+@pytest.mark.parametrize("n", [33, 1025])
+def test_mean_of_an_infinite_potential_is_infinite(n):
+    """A sum that leaves the finite numbers keeps its sign: the centred finite
+    potentials are then -inf, as with a float64 sum."""
+    from paper_2607_11952_gb300 import _lib as L
+    from paper_2607_11952_gb300 import api, gnn
+    graph, m = api.Graph(n, np.zeros((0, 2), np.int64)), gnn.WarmStartModel(gnn.init_params(n))
+    lv, zero = torch.randn(n, device="cuda"), torch.zeros(n, device="cuda")
+    lv[n // 2] = float("inf")
+    F = torch.empty(n, G.FIN, device="cuda")
+    L.fa_gnn_features(graph.handle, lv, zero, zero, zero, 1, F, m.ws(n))
+    want = torch.full((n,), -float("inf"), device="cuda")
+    want[n // 2] = float("nan")
+    torch.testing.assert_close(F[:, 0], want, rtol=0, atol=0, equal_nan=True)
+    assert torch.isfinite(F[:, 1:]).all()
