@@ -437,6 +437,17 @@ fa_status fa_sweep_plan(int32_t n1, int64_t ld, int32_t dtype, int32_t* out);
  * -------------------------------------------------------------------- */
 fa_status fa_ctx_selftest_wait(fa_ctx* ctx, fa_stream_t stream);
 
+/* ----------------------------------------------------------------------
+ * fa_ctx_selftest_solve -- the same for the one-launch solve of small
+ * kernels (see fa_sinkhorn).  In the context's next such solve the CTA
+ * silent_cta (>= 0; -1: none) publishes no partial sums, so that every
+ * CTA's waits run out, after wait_ms (1 to 2000) instead of about 2 s.
+ * That fa_sinkhorn returns FA_ERR_TIMEOUT; nothing is faulted and the
+ * context stays usable.  FA_ERR_UNSUPPORTED where the context's K does not
+ * fit the one-launch solve.  Host state only.
+ * -------------------------------------------------------------------- */
+fa_status fa_ctx_selftest_solve(fa_ctx* ctx, int32_t silent_cta, int32_t wait_ms);
+
 /* Per-thread description of the last error. */
 const char* fa_last_error_string(void);
 

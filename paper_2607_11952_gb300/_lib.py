@@ -93,6 +93,7 @@ SIGNATURES = {
     "fa_sinkhorn_step_static": (_i32, [_p, _i32, _i32, _i32, _i64, _p, _p, _p, _p, _p, _p]),
     "fa_plan_change": (_i32, [_p, _p, _p, _p, _p, _p, _p, _p, _p]),
     "fa_ctx_selftest_wait": (_i32, [_p, _p]),
+    "fa_ctx_selftest_solve": (_i32, [_p, _i32, _i32]),
     "fa_graph_csr_host": (_i32, [_i32, _i64, _p, _p, ctypes.POINTER(_i64), _p, _p, _p, _p,
                                  _i64]),
     "fa_sweep_plan": (_i32, [_i32, _i64, _i32, _p]),
@@ -262,6 +263,10 @@ def fa_sweep_plan(n1: int, ld: int, dtype: int) -> dict:
 
 def fa_ctx_selftest_wait(ctx, stream=None) -> None:
     _check(lib().fa_ctx_selftest_wait(ctx, stream_ptr(stream)), "fa_ctx_selftest_wait")
+
+
+def fa_ctx_selftest_solve(ctx, silent_cta: int, wait_ms: int) -> None:
+    _check(lib().fa_ctx_selftest_solve(ctx, silent_cta, wait_ms), "fa_ctx_selftest_solve")
 
 
 def fa_topk(ctx, K, log_v, k, idx, score, stream=None) -> None:

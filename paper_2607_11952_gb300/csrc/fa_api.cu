@@ -269,7 +269,7 @@ fa_status fa_ctx_create(const fa_graph* g1, const fa_graph* g2,
   SweepPlan sp = plan_sweep(c->n1, c->ld, bf16, 1 << 20);
   int maxact = sp.Q >= 1 ? sweep_max_active_clusters(sp, bf16) : 0;
   c->G_sweep = std::max(1, maxact);
-  c->small_C = solve_small_clusters(c->n1, c->ld, bf16);
+  c->small_G = solve_small_ctas(c->n1, c->ld, bf16);
   c->maxG = std::max(c->G_sweep, normalize_groups(c->n1));
   const int64_t n1 = c->n1, n2 = c->n2, ld = c->ld, ld1 = c->ld1;
   fa_status st;
@@ -292,7 +292,7 @@ fa_status fa_ctx_create(const fa_graph* g1, const fa_graph* g2,
       (st = dalloc(&c->err_part, (size_t)col_finalize_max_blocks((int)n2), acc)) != FA_OK ||
       (st = dalloc(&c->ticket, 1, acc)) != FA_OK ||
       (st = dalloc(&c->result, 1, acc)) != FA_OK ||
-      (st = dalloc(&c->small_words, solve_small_words(c->small_C, c->ld), acc)) != FA_OK ||
+      (st = dalloc(&c->small_words, solve_small_words(c->small_G, c->ld), acc)) != FA_OK ||
       (st = dalloc(&c->diff, (size_t)kPlanDiffBlocks + 1, acc)) != FA_OK) {
     fa_ctx_destroy(c);
     return st;
@@ -301,7 +301,7 @@ fa_status fa_ctx_create(const fa_graph* g1, const fa_graph* g2,
   c->status = &c->result->status;
   if (cudaMemset(c->ticket, 0, sizeof(unsigned)) != cudaSuccess ||
       cudaMemset(c->result, 0, sizeof(SolveResult)) != cudaSuccess ||
-      (c->small_C > 0 && cudaMemset(c->small_words, 0, solve_small_words(c->small_C, c->ld)) != cudaSuccess) ||
+      (c->small_G > 0 && cudaMemset(c->small_words, 0, solve_small_words(c->small_G, c->ld)) != cudaSuccess) ||
       cudaMemset(c->anc_ptr, 0, (n1 + 1) * sizeof(int32_t)) != cudaSuccess ||
       cudaMemset(c->intra1, 0, std::max<int64_t>(1, g1->d.nnz) * sizeof(float)) != cudaSuccess ||
       cudaMemset(c->intra2, 0, std::max<int64_t>(1, g2->d.nnz) * sizeof(float)) != cudaSuccess) {
@@ -556,19 +556,22 @@ fa_status fa_sinkhorn(fa_ctx* c, const void* K, float* log_u, float* log_v,
   // c->status is not cleared here: bits set by earlier asynchronous calls on
   // this context (a bounded wait in the node-cost GEMM, a non-finite row in
   // Pass B) are reported by this call, which clears them once read.
-  const bool small = c->small_C > 0 && !sweep_forced(c);
+  const bool small = c->small_G > 0 && !sweep_forced(c);
   if (small) {
     // every iteration of every solve has a tag of its own; start again (from
     // cleared words) before the 32 bits run out
     if (c->small_tag > UINT32_MAX - (uint32_t)max_iter - 1u) {
-      FA_CUDA(cudaMemsetAsync(c->small_words, 0, solve_small_words(c->small_C, c->ld), s));
+      FA_CUDA(cudaMemsetAsync(c->small_words, 0, solve_small_words(c->small_G, c->ld), s));
       c->small_tag = 0;
     }
     const uint32_t tag0 = c->small_tag;
     c->small_tag += (uint32_t)max_iter;
-    FA_TRY(launch_solve_small(c->small_C, n1, n2, c->ld, K, bf16, warm_log_v ? warm_log_v : log_v,
+    FA_TRY(launch_solve_small(c->small_G, n1, n2, c->ld, K, bf16, warm_log_v ? warm_log_v : log_v,
                               log_u, log_v, max_iter, tol, check_every, c->small_words, tag0,
-                              c->err, &c->result->iters, c->status, s));
+                              c->err, &c->result->iters, c->status, s, c->small_limit_ns,
+                              c->small_silent));
+    c->small_limit_ns = 0;
+    c->small_silent = -1;
     return finish_solve(c, 0, tol, iters_out, err_out, s);
   }
   SweepPlan sp = plan_sweep(n1, c->ld, bf16, c->G_sweep);
@@ -720,6 +723,22 @@ fa_status fa_sweep_plan(int32_t n1, int64_t ld, int32_t dtype, int32_t* out) {
 fa_status fa_ctx_selftest_wait(fa_ctx* c, fa_stream_t stream) {
   if (!c) { set_error("fa_ctx_selftest_wait: NULL ctx"); return FA_ERR_ARG; }
   return launch_wait_selftest(c->status, reinterpret_cast<cudaStream_t>(stream));
+}
+
+fa_status fa_ctx_selftest_solve(fa_ctx* c, int32_t silent_cta, int32_t wait_ms) {
+  if (!c) { set_error("fa_ctx_selftest_solve: NULL ctx"); return FA_ERR_ARG; }
+  if (c->small_G == 0) {
+    set_error("fa_ctx_selftest_solve: this context has no one-launch solve");
+    return FA_ERR_UNSUPPORTED;
+  }
+  if (silent_cta < -1 || silent_cta >= c->small_G || wait_ms < 1 || wait_ms > 2000) {
+    set_error("fa_ctx_selftest_solve: silent_cta=%d (of %d), wait_ms=%d outside [1, 2000]",
+              silent_cta, c->small_G, wait_ms);
+    return FA_ERR_ARG;
+  }
+  c->small_silent = silent_cta;
+  c->small_limit_ns = (uint64_t)wait_ms * 1000000u;
+  return FA_OK;
 }
 
 // ------------------------------------------------------------ plan change

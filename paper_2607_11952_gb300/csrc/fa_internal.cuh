@@ -149,13 +149,16 @@ fa_status launch_sweep(const SweepPlan& sp, int n1, int n2, int64_t ld,
 int sweep_max_active_clusters(const SweepPlan& sp, bool bf16);
 int col_finalize_max_blocks(int n2);
 // one-launch solve of small problems (k_solve_small.cu)
-int solve_small_clusters(int n1, int64_t ld, bool bf16);
+int solve_small_ctas(int n1, int64_t ld, bool bf16);
 // bytes of its exchange words (0 at first); tags grow from one solve to the next
-inline size_t solve_small_words(int C, int64_t ld) { return (size_t)2 * C * ld * 8; }
-fa_status launch_solve_small(int C, int n1, int n2, int64_t ld, const void* K, bool bf16,
+size_t solve_small_words(int G, int64_t ld);
+// limit_ns: of each wait, 0 for the default; silent: a CTA that publishes no
+// partial sums (the failure-detection self-test), -1 for none
+fa_status launch_solve_small(int G, int n1, int n2, int64_t ld, const void* K, bool bf16,
                              const float* log_v_in, float* log_u, float* log_v_out, int max_iter,
                              double tol, int check_every, void* words, uint32_t tag0,
-                             double* err, int* iters, int* status, cudaStream_t s);
+                             double* err, int* iters, int* status, cudaStream_t s,
+                             uint64_t limit_ns = 0, int silent = -1);
 fa_status launch_col_finalize(int n2, int64_t ld, int G, const float* colpart,
                               const float* log_v_cur, float nu,
                               float* log_v_next, double* err_part,
@@ -231,7 +234,9 @@ struct fa_ctx {
   int* status = nullptr;          // = &result->status, the device status word
   char* small_words = nullptr;    // exchange words of the one-launch solve
   uint32_t small_tag = 0;         // tags used so far
-  int small_C = 0;                // its clusters; 0: K does not fit
+  int small_G = 0;                // its CTAs; 0: K does not fit
+  uint64_t small_limit_ns = 0;    // self-test of the next one-launch solve: its
+  int small_silent = -1;          // waits' limit and the CTA that publishes nothing
   int64_t ws_bytes = 0;
   // timing
   int G_sweep = 1;                // co-resident clusters of the sweep
