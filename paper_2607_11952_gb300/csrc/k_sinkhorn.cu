@@ -755,9 +755,12 @@ __global__ void __launch_bounds__(NT, 2) k_sweep_reg(
 template <typename TK, int S, int R>
 static void* sweep_ptr(int NT) {
   // measured (GB300, BF16): only three vectors per thread and two rows per
-  // step are faster with K carried in registers (24,000 columns in clusters
-  // of 4: 0.335 -> 0.290 ms, 12,000 in 2: 74 -> 66 us, 5,000 in 1: 20.7 ->
-  // 18.4 us); one row per step loses 10-17%, four vectors and two rows 8%
+  // step are faster with K carried in registers (12,000 columns in clusters
+  // of 2: 74 -> 66 us, 5,000 in 1: 20.7 -> 18.4 us; forced at 24,000 columns
+  // in clusters of 4 0.335 -> 0.290 ms, where the planner takes clusters of 3
+  // with four vectors instead); one row per step loses 10-17%, four vectors
+  // and two rows 8%.  Planned up to 6,144 columns, around 12,000, 21,000 and
+  // 42,000.
   if constexpr (sizeof(TK) == 2 && S == 3 && R == 2)
     if (NT == 256) return reinterpret_cast<void*>(&k_sweep_reg<TK, S, R, 256>);
   if (NT == 1024) {   // 64 registers per thread: only small slabs per thread
@@ -967,21 +970,29 @@ SweepPlan plan_sweep(int n1, int64_t ld, bool bf16, int max_G) {
   // ld; W is the widest slab.  A step costs a fixed part (barriers, the
   // exchange) plus a part per round of NT vectors, so a shape should have
   // few rounds, a nearly full last round and, where the ring allows, two
-  // rows per step.  BF16 default rule, each line
-  // where the shapes above it do not fit (measured on GB300, fraction of the
-  // copy peak against the rule that began at line 3; 30k-110k columns: lines
-  // 3 to 5 pick the fastest of themselves at every width):
-  //   1. the smallest cluster up to 8 with two rows per step and four or five
-  //      nearly full rounds (88%, 86%): 18k columns 0.65 -> 0.76 (clusters of
-  //      2), 24k 0.64 -> 0.77 (3), 36k 0.70 -> 0.79 (4), 40k 0.71 -> 0.78
-  //      (5), 44k 0.63 -> 0.75 (5); at 50k six CTAs (82% full) tie with line
-  //      4's five, seven (87%) lose;
-  //   2. the smallest cluster of 2 to 4 with two rows and three full rounds
-  //      (95%): 12k 0.58 -> 0.65;
+  // rows per step.  BF16 default rule, each line where the shapes above it do
+  // not fit:
+  //   1. the smallest cluster up to 6 with two rows per step and five rounds
+  //      at least 83.5% full or four at least 88% full;
+  //   2. seven CTAs with two rows and four rounds at least 97% full;
   //   3. the smallest power-of-two cluster up to 8 whose slab takes at most
   //      5 vectors per thread with the last round at least 80% full;
   //   4. the smallest cluster up to 10 with at most 5 vectors;
   //   5. the smallest cluster of any size that fits the register shapes.
+  // Lines 1 and 2 against what lines 3 to 5 take in their place, us per
+  // iteration of 24,000 rows (GB300; clusters x vectors x rows per step):
+  //   21,632-24,576 columns    4x3x2 240 -> 3x4x2 233 (228 below 22,400)
+  //   26,240-27,904            4x4x2 291 -> 3x5x2 259
+  //   37,376-40,960            4x5x1 417 -> 5x4x2 380
+  //   42,752-46,592            8x3x2 493 -> 5x5x2 423
+  //   46,720-49,152            8x3x2 492 -> 6x4x2 476
+  //   52,480-55,808            8x4x2 594 -> 6x5x2 527
+  //   55,936-57,344            8x4x2 593 -> 7x4x2 579
+  // and where they would lose: at 50,560-52,352 seven CTAs (7x4x2, 88-91%
+  // full) 570 to 579 against 532 (5x5x1) and 527 (6x5x2); at 61,696-65,152
+  // 7x5x2 644 against 8x4x2 610; at 17,536 three full rounds (3x3x2) 185
+  // against 2x5x2 169.  30k-110k columns: lines 3 to 5 pick the fastest of
+  // themselves at every width.
   // FP32, already at the copy peak, keeps powers of two.  FA_SWEEP_ANYQ=0
   // forces powers of two, =1 the smallest cluster of any size.
   const int64_t units = ld / V;
@@ -1018,9 +1029,9 @@ SweepPlan plan_sweep(int n1, int64_t ld, bool bf16, int max_G) {
     if (qrule == 2) {
       const int s5 = smax < 5 ? smax : 5;
       if (NT == 256 && smax >= 5) {
-        for (int Q = 1; Q <= 8 && sp.Q == 0; ++Q)
-          if (!fit(Q, min_ns, 5, 0.86, 5, 2)) fit(Q, min_ns, 4, 0.88, 4, 2);
-        for (int Q = 2; Q <= 4 && sp.Q == 0; ++Q) fit(Q, min_ns, 3, 0.95, 3, 2);
+        for (int Q = 1; Q <= 6 && sp.Q == 0; ++Q)
+          if (!fit(Q, min_ns, 5, 0.835, 5, 2)) fit(Q, min_ns, 4, 0.88, 4, 2);
+        if (sp.Q == 0) fit(7, min_ns, 4, 0.97, 4, 2);
       }
       for (int Q = 1; Q <= 8 && sp.Q == 0; Q *= 2) fit(Q, min_ns, s5, 0.8);
       for (int Q = 1; Q <= 10 && sp.Q == 0; ++Q) fit(Q, min_ns, s5, 0.0);
