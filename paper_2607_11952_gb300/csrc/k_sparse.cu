@@ -522,26 +522,6 @@ fa_status launch_spmm_T(const DevGraph& g, int n_cols, int64_t ldd, int64_t ldw,
 __device__ __forceinline__ float to_f32(float v) { return v; }
 __device__ __forceinline__ float to_f32(__nv_bfloat16 v) { return __bfloat162float(v); }
 
-// Natural logarithm of 0 <= x < infinity for the log-kernel: x = 2^e m with m
-// in [0.75, 1.5), log x = e ln 2 + ln 2 lg2(m).  The hardware's lg2 is within
-// 2^-22 absolutely on (0.5, 2), 1.7e-7 in natural units, below the rounding
-// of a result of more than 2 (1.2e-7 to 4e-6 at the |log| of 2 to 90 met
-// here); lg2(1) = 0 exactly, denormals are scaled by 2^23 first, 0 gives
-// -infinity.  The epilogue takes two logarithms per element, and logf was
-// most of its instructions.
-__device__ __forceinline__ float log_pos(float x) {
-  const bool tiny = x < 1.17549435e-38f;
-  const uint32_t b = __float_as_uint(tiny ? x * 8388608.f : x);
-  const int e = (int)(b - 0x3f400000u) >> 23;
-  const float m = __uint_as_float(b - ((uint32_t)e << 23));
-  float l;
-  asm("lg2.approx.f32 %0, %1;" : "=f"(l) : "f"(m));
-  const float r = fmaf((float)(tiny ? e - 23 : e), 0.693147180559945f, l * 0.693147180559945f);
-  return x == 0.f ? -INFINITY : r;
-}
-// negative numbers, infinities and NaN: out of line, never in a valid plan
-__device__ __noinline__ float log_any(float x) { return logf(x); }
-
 template <bool VEC>
 __device__ __forceinline__ float2 load_pair(const float* p) {
   if constexpr (VEC) return __ldcs(reinterpret_cast<const float2*>(p));
@@ -569,8 +549,10 @@ __device__ __forceinline__ float2 load_kernel_pair(const __nv_bfloat16* p) {
 // What bounds it: 512-byte gathers of W^T from L2 (8 nnz2 n1 bytes) and the
 // issue slots of the epilogue (two logarithms per element); HBM moves
 // (16 + b) n1 n2 bytes.  Measured on GB300, 50,000 nodes of degree 10, BF16:
-// 28.9 -> 18.1 ms (200 GB of gathers, 45 GB of HBM); 10,000 nodes FP32: 1.07
-// -> 0.67 ms.  Without its edges the kernel takes 0.3 ms at 10,000 nodes.
+// 28.9 -> 18.7 ms (200 GB of gathers, 45 GB of HBM); 10,000 nodes FP32: 1.07
+// -> 0.69 ms.  logf is 0.6 ms of it: the hardware's lg2 on a split argument
+// took 18.1 ms, but it is off by up to 1.7e-7 absolutely where K is near 1
+// and logf nearly exact.  Without its edges the kernel takes 0.3 ms at 10,000 nodes.
 // 5 CTAs per SM with batches of 2 (48 registers): 20.8 ms; a scan of the
 // row's anchors per element instead of the tile's flag: 19.8 ms.
 constexpr int kRT = 64;    // rows per tile
@@ -726,14 +708,7 @@ __global__ void __launch_bounds__(256, 4) k_spmm_right_cost(
           if (m & 2u) can1 = c_on;
         }
         const float n0 = fmaxf(za.y, ep.delta), n1v = fmaxf(zb.y, ep.delta);
-        float ln0 = log_pos(n0), ln1 = log_pos(n1v), lk0 = log_pos(kp[t].x), lk1 = log_pos(kp[t].y);
-        if ((__float_as_uint(n0) | __float_as_uint(n1v) | __float_as_uint(kp[t].x) |
-             __float_as_uint(kp[t].y)) >= 0x7f800000u) {
-          ln0 = log_any(n0);
-          ln1 = log_any(n1v);
-          lk0 = log_any(kp[t].x);
-          lk1 = log_any(kp[t].y);
-        }
+        const float ln0 = logf(n0), ln1 = logf(n1v), lk0 = logf(kp[t].x), lk1 = logf(kp[t].y);
         const float C0 = cn[t].x + ep.lam_e * za.x - ep.lam_n * ln0 + ep.lam_a * can0;
         const float C1 = cn[t].y + ep.lam_e * zb.x - ep.lam_n * ln1 + ep.lam_a * can1;
         float x0 = -C0 * inv_eps, x1 = -C1 * inv_eps;
