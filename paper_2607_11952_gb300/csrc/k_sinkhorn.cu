@@ -185,7 +185,9 @@ constexpr size_t kSmemBudget = 220 * 1024;
 // which time each receiver has consumed step t-4 (the slot's previous user)
 // and re-armed it, so kNX = 4 slots never alias.  One cluster barrier after
 // the mbarrier initialisation and one before exit bracket all remote
-// traffic; every mbarrier wait is bounded.
+// traffic; every mbarrier wait is bounded.  A CTA whose wait gave up arms and
+// sends nothing more: a barrier whose phase never completed must not be
+// armed again, and its peers' waits then run out in turn.
 // CTAs per SM a launch shape is built for: 256-thread CTAs whose threads own
 // at most 16 elements of a row run four to an SM, wider ones two.
 __host__ __device__ constexpr int sweep_ctas_per_sm(int NT, int elems_per_thread) {
@@ -381,7 +383,7 @@ __global__ void __launch_bounds__(NT, sweep_ctas_per_sm(NT, S * KT<TK>::V)) k_sw
         for (int r = 0; r < R; ++r) rb[r * NW + warp] = p[r];
       }
       __syncthreads();
-      if (Q > 1 && tid < R) {
+      if (Q > 1 && !dead && tid < R) {
         float sum = 0.f;
 #pragma unroll
         for (int w = 0; w < NW; ++w) sum += rb[tid * NW + w];
@@ -471,7 +473,7 @@ __global__ void __launch_bounds__(NT, sweep_ctas_per_sm(NT, S * KT<TK>::V)) k_sw
       __syncthreads();   // stage tp, red[tp & 1] and slot tp % kNX consumed
       dead = s_timeout != 0;
       if (tid == 0) {
-        if (Q > 1 && tp + kNX < T) mbar_expect_tx(smem_u32(&xbar[tp % kNX]), xch_bytes);
+        if (Q > 1 && !dead && tp + kNX < T) mbar_expect_tx(smem_u32(&xbar[tp % kNX]), xch_bytes);
         if (!dead && tp + NS < T) {
           issue(tp + NS, stage);
           issued = tp + NS + 1;
@@ -706,7 +708,7 @@ __global__ void __launch_bounds__(NT, 2) k_sweep_reg(
     }
     __syncthreads();   // row partials of step t; stage t and slot t-1 are consumed
     dead = s_timeout != 0;
-    if (Q > 1 && tid < R) {
+    if (Q > 1 && !dead && tid < R) {
       float sum = 0.f;
 #pragma unroll
       for (int w = 0; w < NW; ++w) sum += rb[tid * NW + w];
@@ -716,7 +718,7 @@ __global__ void __launch_bounds__(NT, 2) k_sweep_reg(
         st_async_f32(map_cluster(slot, (uint32_t)dst), sum, map_cluster(bar, (uint32_t)dst));
     }
     if (tid == kLead) {
-      if (Q > 1 && t > 0 && t - 1 + kNX < T)
+      if (Q > 1 && !dead && t > 0 && t - 1 + kNX < T)
         mbar_expect_tx(smem_u32(&xbar[(t - 1) % kNX]), xch_bytes);
       if (!dead && t + NS < T) {
         issue(t + NS, stage);

@@ -253,7 +253,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) k_sweep_mma(
     }
     __syncthreads();
     // -------- exchange the CTA's partial row sums within the cluster
-    if (Q > 1 && warp == 0) {
+    if (Q > 1 && !dead && warp == 0) {
       float rs = 0.f;
 #pragma unroll
       for (int w = 0; w < NW; ++w) rs += red[w * R8 + (lane & 7)];
@@ -316,7 +316,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) k_sweep_mma(
     __syncthreads();   // stage, red and exchange slot consumed
     dead = s_timeout != 0;
     if (tid == 0) {
-      if (Q > 1 && t + kNXm < T) mbar_expect_tx(smem_u32(&xbar[t % kNXm]), xch_bytes);
+      if (Q > 1 && !dead && t + kNXm < T) mbar_expect_tx(smem_u32(&xbar[t % kNXm]), xch_bytes);
       if (!dead && t + NS < T) {
         issue(t + NS, stage);
         issued = t + NS + 1;
