@@ -443,8 +443,10 @@ fa_status fa_ctx_selftest_wait(fa_ctx* ctx, fa_stream_t stream);
  * silent_cta (>= 0; -1: none) publishes no partial sums, so that every
  * CTA's waits run out, after wait_ms (1 to 2000) instead of about 2 s.
  * That fa_sinkhorn returns FA_ERR_TIMEOUT; nothing is faulted and the
- * context stays usable.  FA_ERR_UNSUPPORTED where the context's K does not
- * fit the one-launch solve.  Host state only.
+ * context stays usable.  silent_cta = -2 instead makes that solve ask for more
+ * CTAs than the device holds; the launch is refused and fa_sinkhorn iterates
+ * with the sweep.  FA_ERR_UNSUPPORTED where the context's K does not fit the
+ * one-launch solve.  Host state only.
  * -------------------------------------------------------------------- */
 fa_status fa_ctx_selftest_solve(fa_ctx* ctx, int32_t silent_cta, int32_t wait_ms);
 

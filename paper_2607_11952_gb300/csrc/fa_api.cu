@@ -566,13 +566,16 @@ fa_status fa_sinkhorn(fa_ctx* c, const void* K, float* log_u, float* log_v,
     }
     const uint32_t tag0 = c->small_tag;
     c->small_tag += (uint32_t)max_iter;
-    FA_TRY(launch_solve_small(c->small_G, n1, n2, c->ld, K, bf16, warm_log_v ? warm_log_v : log_v,
+    const fa_status st = launch_solve_small(c->small_G, n1, n2, c->ld, K, bf16, warm_log_v ? warm_log_v : log_v,
                               log_u, log_v, max_iter, tol, check_every, c->small_words, tag0,
                               c->err, &c->result->iters, c->status, s, c->small_limit_ns,
-                              c->small_silent));
+                              c->small_silent);
     c->small_limit_ns = 0;
     c->small_silent = -1;
-    return finish_solve(c, 0, tol, iters_out, err_out, s);
+    if (st == FA_OK) return finish_solve(c, 0, tol, iters_out, err_out, s);
+    if (st != FA_ERR_UNSUPPORTED) return st;
+    // the device does not hold all CTAs at once now: the sweeps need no more
+    // than one cluster resident
   }
   SweepPlan sp = plan_sweep(n1, c->ld, bf16, c->G_sweep);
   if (warm_log_v)
@@ -731,7 +734,7 @@ fa_status fa_ctx_selftest_solve(fa_ctx* c, int32_t silent_cta, int32_t wait_ms) 
     set_error("fa_ctx_selftest_solve: this context has no one-launch solve");
     return FA_ERR_UNSUPPORTED;
   }
-  if (silent_cta < -1 || silent_cta >= c->small_G || wait_ms < 1 || wait_ms > 2000) {
+  if (silent_cta < -2 || silent_cta >= c->small_G || wait_ms < 1 || wait_ms > 2000) {
     set_error("fa_ctx_selftest_solve: silent_cta=%d (of %d), wait_ms=%d outside [1, 2000]",
               silent_cta, c->small_G, wait_ms);
     return FA_ERR_ARG;

@@ -153,7 +153,9 @@ int solve_small_ctas(int n1, int64_t ld, bool bf16);
 // bytes of its exchange words (0 at first); tags grow from one solve to the next
 size_t solve_small_words(int G, int64_t ld);
 // limit_ns: of each wait, 0 for the default; silent: a CTA that publishes no
-// partial sums (the failure-detection self-test), -1 for none
+// partial sums (the failure-detection self-test), -1 for none, -2 for a launch
+// that is refused.  FA_ERR_UNSUPPORTED: not launched, the device does not hold
+// the CTAs at once.
 fa_status launch_solve_small(int G, int n1, int n2, int64_t ld, const void* K, bool bf16,
                              const float* log_v_in, float* log_u, float* log_v_out, int max_iter,
                              double tol, int check_every, void* words, uint32_t tag0,

@@ -386,11 +386,17 @@ fa_status launch_solve_small(int G, int n1, int n2, int64_t ld, const void* K, b
                   (void*)&log_v_out, (void*)&mu, (void*)&log_mu, (void*)&nu, (void*)&max_iter,
                   (void*)&tol, (void*)&check_every, (void*)&words, (void*)&tag0, (void*)&err,
                   (void*)&iters, (void*)&status, (void*)&limit_ns, (void*)&silent};
-  cudaError_t e = cudaLaunchCooperativeKernel(fn, dim3((unsigned)G), dim3(kST), args, smem, s);
+  // self-test -2: more CTAs than any device holds, which the runtime refuses
+  const int ask = silent == -2 ? 1 << 20 : G;
+  cudaError_t e = cudaLaunchCooperativeKernel(fn, dim3((unsigned)ask), dim3(kST), args, smem, s);
   if (e != cudaSuccess) {
-    set_error("k_solve_small launch (%d CTAs, %zu bytes): %s", G, smem, cudaGetErrorString(e));
+    set_error("k_solve_small launch (%d CTAs, %zu bytes): %s", ask, smem, cudaGetErrorString(e));
     cudaGetLastError();
-    return FA_ERR_CUDA;
+    // refused, not failed: the caller has another way
+    return e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorLaunchOutOfResources ||
+                   e == cudaErrorNotSupported
+               ? FA_ERR_UNSUPPORTED
+               : FA_ERR_CUDA;
   }
   FA_LAUNCHED("k_solve_small");
   return FA_OK;
