@@ -256,16 +256,21 @@ fa_status launch_rank(int n2, int64_t ld, const void* K, bool bf16,
 // ------------------------------------------------------------ plan change
 // sum_ij |T_a,ij - T_b,ij| with T = diag(exp(log_u)) K diag(exp(log_v)):
 // each element's two plan values in float32, their absolute differences
-// summed with at least float64's care in a fixed order: every thread keeps
-// its sum as an unevaluated pair of floats (Knuth's two-sum: hi + lo carries
-// about 48 bits), widened to float64 once at the end, because one float64
-// add per element would be bound by this GPU's few float64 units.  A thread
-// owns V = 4 or 8 columns (their scalings in registers) of the rows
-// blockIdx.y, + gridDim.y, ...; the block sums are added by one block in a
-// fixed tree.  Bound by the two reads of K.  5,000 x 5,000 BF16: 130 us with
-// an exponential and a float64 add per element plus 52 us for a one-thread
-// final sum; 31.5 us and about 3 us now.
+// summed in float64 in a fixed order.  One float64 add per element would be
+// bound by this GPU's few float64 units, so a thread sums kDiffRows rows of
+// its V = 4 or 8 columns as two unevaluated pairs of floats (Knuth's two-sum,
+// at most 32 terms each) and adds the pairs to its float64 sum; a group whose
+// float sum is not finite is summed again in float64.  Over 1,600
+// random sums of 24 to 1,568 terms a thread's sum is off by at most one unit
+// of float64 (1.1e-16 relative).  A thread owns V columns (their scalings in
+// registers) of the rows blockIdx.y, + gridDim.y, ...; the block sums are
+// added by one block in a fixed tree.  Bound by the two reads of K.  Whole
+// call with its read-back, against an exponential and a float64 add per
+// element and a one-thread final sum: 5,000 x 5,000 BF16 206 -> 67 us, 20,000
+// 1,990 -> 384 us (374 us with one float pair per thread, which holds only
+// float32's range; 438 with 4 rows a group).
 constexpr int kDiffThreads = 256;
+constexpr int kDiffRows = 8;
 
 __device__ __forceinline__ void two_sum_add(float& hi, float& lo, float x) {
   const float s = __fadd_rn(hi, x);
@@ -281,7 +286,7 @@ __global__ void __launch_bounds__(kDiffThreads) k_plan_l1diff(
     const float* __restrict__ lvb, double* __restrict__ part) {
   constexpr int V = RowVec<TK>::V;
   __shared__ double red[kDiffThreads / 32];
-  float hi[2] = {0.f, 0.f}, lo[2] = {0.f, 0.f};
+  double acc = 0.0;
   for (int64_t jb = ((int64_t)blockIdx.x * kDiffThreads + threadIdx.x) * V; jb < n2;
        jb += (int64_t)gridDim.x * kDiffThreads * V) {
     const int j0 = (int)jb;
@@ -291,8 +296,7 @@ __global__ void __launch_bounds__(kDiffThreads) k_plan_l1diff(
       va[e] = j0 + e < n2 ? expf(lva[j0 + e]) : 0.f;
       vb[e] = j0 + e < n2 ? expf(lvb[j0 + e]) : 0.f;
     }
-#pragma unroll 2
-    for (int i = blockIdx.y; i < n1; i += gridDim.y) {
+    auto row = [&](int i, auto&& add) {      // |T_a - T_b| of row i to add(e, .)
       const int64_t at = (int64_t)i * ld + j0;
       float ka[V], kb[V];
       widen(load_row16<TK, VEC>(Ka + at), ka, TK());
@@ -302,12 +306,24 @@ __global__ void __launch_bounds__(kDiffThreads) k_plan_l1diff(
       for (int e = 0; e < V; ++e) {
         const float ta = __fmul_rn(__fmul_rn(ua, ka[e]), va[e]);
         const float tb = __fmul_rn(__fmul_rn(ub, kb[e]), vb[e]);
-        const float d = fabsf(ta - tb);
-        two_sum_add(hi[e & 1], lo[e & 1], j0 + e < n2 ? d : 0.f);
+        add(e, j0 + e < n2 ? fabsf(ta - tb) : 0.f);
       }
+    };
+    for (int i0 = blockIdx.y; i0 < n1; i0 += kDiffRows * gridDim.y) {
+      float hi[2] = {0.f, 0.f}, lo[2] = {0.f, 0.f};
+#pragma unroll 4
+      for (int i = i0; i < min(n1, i0 + kDiffRows * (int)gridDim.y); i += gridDim.y)
+        row(i, [&](int e, float d) { two_sum_add(hi[e & 1], lo[e & 1], d); });
+      double t = ((double)hi[0] + (double)hi[1]) + ((double)lo[0] + (double)lo[1]);
+      if (!isfinite(hi[0] + hi[1])) {        // beyond float32's range, or not finite at all
+        t = 0.0;
+#pragma unroll 1
+        for (int i = i0; i < min(n1, i0 + kDiffRows * (int)gridDim.y); i += gridDim.y)
+          row(i, [&](int, float d) { t += (double)d; });
+      }
+      acc += t;
     }
   }
-  double acc = ((double)hi[0] + (double)hi[1]) + ((double)lo[0] + (double)lo[1]);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
