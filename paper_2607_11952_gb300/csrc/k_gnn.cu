@@ -25,7 +25,6 @@ constexpr int kOffW2 = kOffB1 + kHid;
 constexpr int kOffC = kOffW2 + kHid;
 
 // workspace (floats): AF n*kFin | A1 n*64 | z2 n | g n | partials nb*kNP | scal 8
-// (and n spare)
 struct GnnWs {
   float *AF, *A1, *z2, *g, *part, *scal;
   int nb;
@@ -47,7 +46,7 @@ static GnnWs ws_layout(float* w, int n) {
   return s;
 }
 int64_t gnn_workspace_floats(int n) {
-  return (int64_t)n * (kFin + kHid + 3) + (int64_t)grad_blocks(n) * kNP + 8;
+  return (int64_t)n * (kFin + kHid + 2) + (int64_t)grad_blocks(n) * kNP + 8;
 }
 
 // ------------------------------------------------------------ reductions

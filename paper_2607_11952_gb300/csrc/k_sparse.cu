@@ -80,10 +80,6 @@ fa_status launch_edge_records(const DevGraph& g, const float* va, const float* v
   return FA_OK;
 }
 
-// A value every lane of the warp holds alike, in a form that the compiler
-// knows to be so: branches on it need no reconvergence code.
-__device__ __forceinline__ int uniform(int v) { return v; }
-
 __device__ __forceinline__ EdgeRec lds_edge(const EdgeRec* p) {
   const int4 v = *reinterpret_cast<const int4*>(p);
   return EdgeRec{v.x, v.y, __int_as_float(v.z), __int_as_float(v.w)};
@@ -193,7 +189,7 @@ __global__ void __launch_bounds__(32 * NW, MINB) k_spmm(
   __shared__ int head_row[NW];
   const int i0 = blockIdx.x * TI;
   const int j0 = blockIdx.y * TJ;
-  const int warp = uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
+  const int warp = (int)threadIdx.x >> 5, lane = threadIdx.x & 31;
   unsigned char* mine = sm_raw + warp * Sh::kWarpBytes;
   for (int t = threadIdx.x; t <= TI; t += 32 * NW) rps[t] = rp[min(i0 + t, n)];
   int cur = -1, cnt, eb;
@@ -216,8 +212,8 @@ __global__ void __launch_bounds__(32 * NW, MINB) k_spmm(
   };
   {
     const int E0 = rp[i0], len = rp[min(i0 + TI, n)] - E0;
-    eb = uniform(E0 + (int)((int64_t)len * warp / NW));
-    const int ee = uniform(E0 + (int)((int64_t)len * (warp + 1) / NW));
+    eb = E0 + (int)((int64_t)len * warp / NW);
+    const int ee = E0 + (int)((int64_t)len * (warp + 1) / NW);
     cnt = ee - eb;
     // a lane past the operand's last column gathers the panel's first ones;
     // its results are never stored
@@ -519,9 +515,6 @@ fa_status launch_spmm_T(const DevGraph& g, int n_cols, int64_t ldd, int64_t ldw,
 // stored as float32, plus the per-(row, 64-column tile) maximum of x, with
 // Z[i, j] = sum_l P2[j, l] s_l W^T[l, i] for both value sets (recs: P2's
 // records, W^T pairs interleaved).
-__device__ __forceinline__ float to_f32(float v) { return v; }
-__device__ __forceinline__ float to_f32(__nv_bfloat16 v) { return __bfloat162float(v); }
-
 template <bool VEC>
 __device__ __forceinline__ float2 load_pair(const float* p) {
   if constexpr (VEC) return __ldcs(reinterpret_cast<const float2*>(p));
@@ -570,7 +563,7 @@ __global__ void __launch_bounds__(256, 4) k_spmm_right_cost(
   __shared__ uint32_t anc[kRT][2];                    // anchors of a row: bit per column
   __shared__ float lus[kRT];
   const int j0 = blockIdx.x * kCT, i0 = blockIdx.y * kRT;
-  const int warp = uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
+  const int warp = (int)threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x <= kCT) rps[threadIdx.x] = rp[min(j0 + (int)threadIdx.x, n2)];
   if (threadIdx.x >= 128 && threadIdx.x < 128 + kRT) {
     // few tiles hold an anchor at all: one flag per tile, a bit per column
@@ -595,8 +588,8 @@ __global__ void __launch_bounds__(256, 4) k_spmm_right_cost(
   };
   {
     const int E0 = rp[min(j0, n2)], len = rp[min(j0 + kCT, n2)] - E0;
-    eb = uniform(E0 + (int)((int64_t)len * warp / 8));
-    const int ee = uniform(E0 + (int)((int64_t)len * (warp + 1) / 8));
+    eb = E0 + (int)((int64_t)len * warp / 8);
+    const int ee = E0 + (int)((int64_t)len * (warp + 1) / 8);
     cnt = ee - eb;
     const char* wrow = reinterpret_cast<const char*>(Wt + (int64_t)(i0 + 2 * lane) * 2);
     const uint32_t ldb = (uint32_t)(ldw * 8);
