@@ -168,11 +168,19 @@ fa_status fa_align_iter(fa_ctx* ctx, void* K, float* log_u, float* log_v,
 
 /* ----------------------------------------------------------------------
  * fa_sinkhorn -- Phase 3 of Algorithm 1 (Eq. 3) on a fixed kernel K.
- * One fused sweep per iteration reads K once: the row update
- * u_i = mu_i / sum_j K_ij v_j (b update) and, in the same pass, the column
- * sums sum_i K_ij u_i for the next column update (a update).  The L1
- * marginal error |T^T 1 - nu|_1 of the plan after each b update is
+ * An iteration is the row update u_i = mu_i / sum_j K_ij v_j (b update) and
+ * the column sums sum_i K_ij u_i for the next column update (a update).  The
+ * L1 marginal error |T^T 1 - nu|_1 of the plan after each b update is
  * computed in FP64 on the device.
+ * Where K fits the SMs' shared memory together (ld <= 4096 and up to about
+ * 2,600 x 2,600 in FP32, 3,600 x 3,600 in BF16) the whole solve is one
+ * cooperative launch that keeps K there and tests the tolerance itself.
+ * Otherwise, and where the device cannot hold that launch at once, while
+ * timing is on (fa_ctx_set_timing) or while any FA_SWEEP_* variable is set, an
+ * iteration is one fused sweep that reads K once and a column finalisation,
+ * and the tolerance is tested on the host.  The two agree up to FP32
+ * summation order and the rounding of log v, which the sweeps carry between
+ * iterations, not bit for bit.
  * In: log_v holds the current column scaling (a_1 from fa_align_iter) unless
  *     warm_log_v (device n2 float32, nullable) is given, which replaces it.
  * Runs until err <= tol at a checked iteration (every check_every
@@ -216,7 +224,9 @@ fa_status fa_rank(fa_ctx* ctx, const void* K, const float* log_v,
 /* ----------------------------------------------------------------------
  * Kernel-level timing of the last fa_sinkhorn call: average device time of
  * one fused sweep (ms), measured with CUDA events on the call's stream
- * when enabled by fa_ctx_set_timing(ctx, 1).
+ * when enabled by fa_ctx_set_timing(ctx, 1).  With timing on, fa_sinkhorn
+ * always iterates with the sweep, also where it would otherwise solve in one
+ * launch (results then differ by rounding), and its launches do not overlap.
  * -------------------------------------------------------------------- */
 fa_status fa_ctx_set_timing(fa_ctx* ctx, int32_t on);
 fa_status fa_ctx_last_sweep_ms(const fa_ctx* ctx, double* ms, int32_t* n);
@@ -302,7 +312,8 @@ fa_status fa_gnn_warm_start(int32_t n, const float* log_v1, const float* pred,
  * correlation of p and y, so that a prediction that explains little of y
  * is trusted little: 1 -> a rho^2, 2 -> a |rho|, anything else -> a.
  * Centred because potentials are defined up to a constant.  pred, y: device vectors of n floats; scale: device scalar.
- * Fixed-order FP64 sums.  Used after each solve to damp the next solve's
+ * Fixed-order sums in pairs of FP32 (about 48 bits), in FP64 over threads
+ * and where the values would leave FP32's range.  Used after each solve to damp the next solve's
  * prediction by how well the last one matched (0: the previous-correction
  * start, 1: the network's own prediction). */
 fa_status fa_gnn_fit_scale(int32_t n, const float* pred, const float* y, float max_abs,
@@ -342,7 +353,8 @@ fa_status fa_plan_change(fa_ctx* ctx, const void* K_a, const float* log_u_a,
  * plan (log_u, log_v) into *err (device double), with mu = 1/n1 and
  * nu = 1/n2.  The partial column sums may be grouped over fewer row groups
  * than fa_sinkhorn uses (the static array bounds them), so results agree
- * with fa_sinkhorn up to FP32 summation order, not bit for bit.
+ * with fa_sinkhorn up to FP32 summation order (and, where fa_sinkhorn solves
+ * in one launch, the rounding of log v), not bit for bit.
  * K: device, n1 x ld, FA_F32 or FA_BF16 (dtype), 16-byte aligned, padding
  * columns 0; log_v, log_u, log_v_next, err: device.
  * status (device int32, nullable) receives the kernels' status bits
