@@ -80,10 +80,11 @@ __device__ __forceinline__ void load_floats(const float* __restrict__ x, int j, 
 // only the compare.  A candidate is inserted by a ballot (its position) and
 // one shuffle; for n columns in no particular order about k (1 + ln(n/k))
 // candidates pass.  Empty entries are (-inf, -1): -inf and NaN scores are
-// never taken.  Bound by the read of K; the widening, the product with v and
-// the maximum are about 1.2 instructions per element.  The form it replaced
-// (one CTA per row, 2-byte loads, a sorted 16-entry list per thread): top-10
-// of 20,000 x 20,000 BF16 in 4.44 ms; this one 0.237 ms (floor 0.12 ms).
+// never taken.  The read of K at half the copy rate; the widening, the
+// product with v and the maximum are about 1.2 instructions per element.  The
+// form it replaced (one CTA per row, 2-byte loads, a sorted 16-entry list per
+// thread): top-10 of 20,000 x 20,000 BF16 in 4.44 ms; this one 0.237 ms (the
+// read alone 0.12 ms).
 template <typename TK, bool VEC>
 __global__ void __launch_bounds__(kTopkThreads) k_topk(
     int n1, int n2, int64_t ld, const TK* __restrict__ K, const float* __restrict__ v,
